@@ -156,9 +156,11 @@ typedef struct {
                               units of every level (for small coarse problems). >= 0 */
     int32_t full_operators; /* 1: store the symmetric local operators in full. 0 (default):
                               in the FP32 and BF16 forms on the CUDA cores with
-                              nrhs_max = 1, A_II^-1 and K_GG are stored as their lower
+                              nrhs_max = 1, and in the FP64 form (as 58-bit block fixed
+                              point, unless an operator has about 3900 rows or more),
+                              A_II^-1 and K_GG are stored as their lower
                               triangles (about half the bytes) and applied by the
-                              symmetric streamed GEMV; elsewhere in full */
+                              symmetric streamed kernels; elsewhere in full */
     int32_t history;       /* PCG iterations whose scalars (||r_k||, alpha_k, beta_k) the
                               handle keeps for bddc_pcg_history, 0..100000; 0 = none */
     int32_t coarse_cg_maxit; /* BDDC_COARSE_CG: iteration limit of the coarse CG, >= 0;

@@ -325,6 +325,8 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
     return upload(h, reinterpret_cast<__nv_bfloat16**>(dst), a);
   };
   int64_t opbytes_I = 0, opbytes_G = 0;
+  const int max_dim = std::max(dIop.empty() ? 0 : *std::max_element(dIop.begin(), dIop.end()),
+                               dG.empty() ? 0 : *std::max_element(dG.begin(), dG.end()));
   if (h->use_tc) {
     // tensor-core path: operators in the MMA tile layout, no row-major copy
     auto up_tc = [&](auto tag, const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
@@ -367,17 +369,23 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
     h->allocations.push_back(pB);
     h->d_tcB = pB;
     h->use_tma = false;
-  } else if (!h->full_operators && h->nrhs_max == 1 && (prec == BDDC_PREC_FP32 || prec == BDDC_PREC_BF16) &&
-             sgemv_tma_supported(prec, std::max(dIop.empty() ? 0 : *std::max_element(dIop.begin(), dIop.end()),
-                                                dG.empty() ? 0 : *std::max_element(dG.begin(), dG.end())))) {
-    // symmetric operators, one right-hand side: lower triangles, one work
-    // item per operator (largest first)
+  } else if (!h->full_operators && (prec == BDDC_PREC_FP64 ? fx_gemm_supported(max_dim)
+                                                           : h->nrhs_max == 1 && sgemv_tma_supported(prec, max_dim))) {
+    // symmetric operators (float32 and bfloat16: one right-hand side): lower
+    // triangles, one work item per operator (largest first)
     auto up_sym = [&](const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
                       const std::vector<int32_t>& voff, void** arena, WorkItem** items, int* n_items, int* max_n,
-                      int64_t* bytes) -> cudaError_t {
+                      int64_t* bytes, int32_t** rexp) -> cudaError_t {
       std::vector<int64_t> off;
       cudaError_t e;
-      if (prec == BDDC_PREC_FP32) {
+      if (prec == BDDC_PREC_FP64) {
+        std::vector<int2> a;
+        std::vector<int32_t> re;
+        fx_pack_lower(ops, dims, voff, hs.threads, off, a, re);
+        arena_bytes += a.size() * sizeof(int2);
+        e = upload(h, reinterpret_cast<int2**>(arena), a);
+        if (e == cudaSuccess) e = upload(h, rexp, re);
+      } else if (prec == BDDC_PREC_FP32) {
         auto a = pack_lower<float>(ops, dims, prec, off, cvt_f);
         arena_bytes += a.size() * sizeof(float);
         e = upload(h, reinterpret_cast<float**>(arena), a);
@@ -393,7 +401,7 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
       for (size_t s = 0; s < dims.size(); ++s) {
         if (dims[s] == 0) continue;
         it.push_back(WorkItem{off[s], padded_ld(dims[s], elem_bytes(prec)), dims[s], 0, dims[s], voff[s], voff[s]});
-        *bytes += sym_packed_elems(prec, dims[s]) * elem_bytes(prec);
+        *bytes += (prec == BDDC_PREC_FP64 ? fx_packed_elems(dims[s]) : sym_packed_elems(prec, dims[s])) * elem_bytes(prec);
         *max_n = std::max(*max_n, dims[s]);
       }
       std::stable_sort(it.begin(), it.end(), [](const WorkItem& a, const WorkItem& b) { return a.ncols > b.ncols; });
@@ -401,11 +409,13 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
       return upload(h, items, it);
     };
     CUDA_TRY(up_sym(hs.AIIinv, dIop, ioff, reinterpret_cast<void**>(&h->d_aii), &h->d_wsy_I, &h->n_wsy_I,
-                    &h->max_n_I, &opbytes_I));
+                    &h->max_n_I, &opbytes_I, &h->d_rexp_I));
     CUDA_TRY(up_sym(hs.Kgg, dG, goff, reinterpret_cast<void**>(&h->d_kgg), &h->d_wsy_G, &h->n_wsy_G, &h->max_n_G,
-                    &opbytes_G));
-    h->use_sym = true;
-    h->use_tma = true;
+                    &opbytes_G, &h->d_rexp_G));
+    h->use_fx = prec == BDDC_PREC_FP64;
+    if (opbytes_I) h->fx_share[0] = 8.0 * fx_packed_elems(h->max_n_I) / opbytes_I;
+    if (opbytes_G) h->fx_share[1] = 8.0 * fx_packed_elems(h->max_n_G) / opbytes_G;
+    h->use_sym = h->use_tma = !h->use_fx;
   } else {
     CUDA_TRY(up_arena(hs.AIIinv, dIop, offI, ldI, &h->d_aii));
     CUDA_TRY(up_arena(hs.Kgg, dG, offG, ldG, &h->d_kgg));
@@ -630,7 +640,7 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
   in.interior_factor_entries = ifac_entries;
   in.interface_op_bytes = opbytes_G;
   in.tensor_cores = h->use_tc ? 1 : 0;
-  in.symmetric_operators = h->use_sym ? 1 : 0;
+  in.symmetric_operators = h->use_sym || h->use_fx ? 1 : 0;
   in.n_interface_copies = h->nG_tot;
   in.coarse_factor_entries = h->c_nnz;
   in.coarse_update_total = h->cs.update_total;

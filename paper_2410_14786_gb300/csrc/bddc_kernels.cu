@@ -532,6 +532,13 @@ cudaError_t local_op(bddc_handle_s* h, bool interior, const double* X, double* Y
                      cudaStream_t st, int max_per_sm = 0) {
   if (interior && h->sparse_local) return interior_sweeps(h, h->w, X, Y, yscatter, nrhs, st);
   if (h->use_tc) return launch_tc_gemm(h, interior, X, Y, yscatter, nrhs, st);
+  if (h->use_fx) {
+    h->launches += (interior ? h->n_wsy_I : h->n_wsy_G) > 0;
+    return interior ? launch_fx_gemm(h->d_wsy_I, h->n_wsy_I, h->max_n_I, h->fx_share[0], h->d_aii, h->d_rexp_I, X, Y,
+                                     yscatter, nrhs, h->d_err, st)
+                    : launch_fx_gemm(h->d_wsy_G, h->n_wsy_G, h->max_n_G, h->fx_share[1], h->d_kgg, h->d_rexp_G, X, Y,
+                                     yscatter, nrhs, h->d_err, st);
+  }
   if (h->use_sym) {
     if (nrhs != 1) return cudaErrorInvalidValue;   // nrhs_max is 1 on this path
     h->launches += (interior ? h->n_wsy_I : h->n_wsy_G) > 0;
@@ -631,7 +638,8 @@ cudaError_t launch_apply(bddc_handle_s* h, const double* r, double* z, int nrhs,
   // grid must be resident). Registers decide the cap: a symmetric-GEMV block
   // holds 288 x 72 and a 256-thread sweep block 256 x 128 of the SM's 65536,
   // so one of the former fits beside the latter; a streamed-GEMV block
-  // (288 x 56) fits twice.
+  // (288 x 56) fits twice. (A block of the float64 fixed-point kernel fills its
+  // SM: there the sweeps start when the interface operator's blocks leave.)
   const int ax = h->aux_sel;
   const bool overlap = h->tune_overlap && h->nG_tot && h->n_c && !h->coarse_dense && h->aux_stream[ax];
   const int cap = h->use_sym ? 1 : 2;

@@ -116,6 +116,7 @@ int host_setup(const bddc_problem_t* P, const bddc_options_t* O, HostSetup& hs, 
   const int nloc = 1 << dim;
   const int maxs = nloc;     // a node touches at most 2^dim elements
   int threads = O->n_threads > 0 ? O->n_threads : (int)std::max(1u, std::thread::hardware_concurrency());
+  hs.threads = threads;
   uint32_t mask = O->constraints ? O->constraints : (BDDC_CORNERS | BDDC_EDGES | BDDC_FACES);
 
   auto node_id = [&](int64_t ix, int64_t iy, int64_t iz) { return ix + n1 * (iy + n1 * iz); };

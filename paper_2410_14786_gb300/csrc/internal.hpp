@@ -336,6 +336,7 @@ struct HostSetup {
   bool sparse_local = false;
   std::vector<CoarseFactor> ifac;
   int error_subdomain = -1;
+  int threads = 1;                           // host threads of the setup
 };
 
 // The work vectors of one apply (each nrhs columns wide, right-hand side
@@ -465,10 +466,15 @@ struct bddc_handle_s {
   bool use_tma = false;
   // symmetric operators as packed lower triangles (one work item per operator)
   bool use_sym = false;
+  bool use_fx = false;                // float64: the same in block fixed point (any number of columns)
   bool full_operators = false;        // option: keep them in full
   bddc::WorkItem* d_wsy_I = nullptr; int n_wsy_I = 0;
   bddc::WorkItem* d_wsy_G = nullptr; int n_wsy_G = 0;
   int max_n_I = 0, max_n_G = 0;
+  // float64: entries in block fixed point, with the exponent of every row
+  // (compact interior / interface numbering)
+  int32_t *d_rexp_I = nullptr, *d_rexp_G = nullptr;
+  double fx_share[2] = {0, 0};        // the largest operator's part of all entries: interior, interface
   // tensor-core path: tiled arenas (d_aii / d_kgg then hold the tiled layout)
   bool use_tc = false;
   bddc::TcUnit* d_tcu_I = nullptr; int n_tcu_I = 0;
