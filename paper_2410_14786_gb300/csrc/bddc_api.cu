@@ -379,11 +379,13 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
       std::vector<int64_t> off;
       cudaError_t e;
       if (prec == BDDC_PREC_FP64) {
-        std::vector<int2> a;
+        std::unique_ptr<int2[]> a;
+        int64_t elems = 0;
         std::vector<int32_t> re;
-        fx_pack_lower(ops, dims, voff, hs.threads, off, a, re);
-        arena_bytes += a.size() * sizeof(int2);
-        e = upload(h, reinterpret_cast<int2**>(arena), a);
+        fx_pack_lower(ops, dims, voff, hs.threads, off, a, elems, re);
+        arena_bytes += elems * sizeof(int2);
+        e = dev_alloc(h, reinterpret_cast<int2**>(arena), elems);
+        if (e == cudaSuccess) e = cudaMemcpy(*arena, a.get(), elems * sizeof(int2), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = upload(h, rexp, re);
       } else if (prec == BDDC_PREC_FP32) {
         auto a = pack_lower<float>(ops, dims, prec, off, cvt_f);

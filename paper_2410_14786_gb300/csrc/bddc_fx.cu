@@ -46,6 +46,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <memory>
 #include <thread>
 #include <vector>
 
@@ -422,76 +423,104 @@ bool fx_gemm_supported(int max_n) {
   return max_n <= kFxMaxBlocks * kFxTile && FxSmem(max_n, 1).total(1) <= (size_t)kFxSmemCap;
 }
 
-void fx_row_scales(const double* A, int n, int32_t* e) {
-  // |a_ij| < 2^(e_i + e_j): from the diagonal, raised where rounding (or a
+// S = (A + A^T) / 2 by tiles (the transposed reads stay in cache), row-major.
+static void fx_symmetric_part(const double* A, int n, double* S) {
+  for (int i0 = 0; i0 < n; i0 += kFxTile)
+    for (int j0 = 0; j0 <= i0; j0 += kFxTile)
+      for (int i = i0; i < std::min(n, i0 + kFxTile); ++i)
+        for (int j = j0; j < std::min(n, j0 + kFxTile); ++j) {
+          const double v = 0.5 * (A[(size_t)i * n + j] + A[(size_t)j * n + i]);
+          S[(size_t)i * n + j] = v;
+          S[(size_t)j * n + i] = v;
+        }
+}
+
+// Row exponents of the symmetric S.
+static void fx_row_scales(const double* S, int n, int32_t* e) {
+  // |s_ij| < 2^(e_i + e_j): from the diagonal, raised where rounding (or a
   // row that vanishes in exact arithmetic) breaks the bound of the semidefinite case
   auto exponent = [](double v) {
     uint64_t b;
     std::memcpy(&b, &v, 8);
     return fx_exponent(b);
   };
-  auto entry = [&](int i, int j) { return std::fabs(0.5 * (A[(size_t)i * n + j] + A[(size_t)j * n + i])); };
   for (int i = 0; i < n; ++i) {
-    const double d = A[(size_t)i * n + i];
+    const double d = S[(size_t)i * n + i];
     e[i] = d != 0.0 ? (exponent(d) + 2049) / 2 - 1024 : -400;
   }
-  for (int i = 0; i < n; ++i)
+  std::vector<double> inv(n), size(n);
+  for (int i = 0; i < n; ++i) size[i] = std::ldexp(1.0, e[i]);
+  for (int i = 0; i < n; ++i) {
+    const double* row = S + (size_t)i * n;
     for (int j = 0; j < i; ++j) {
-      const int need = exponent(entry(i, j)) - e[i] - e[j];
-      if (need > 0) (e[i] < e[j] ? e[i] : e[j]) += need;
+      if (std::fabs(row[j]) < size[i] * size[j]) continue;   // the common case
+      const int need = exponent(row[j]) - e[i] - e[j];
+      if (need <= 0) continue;
+      const int up = e[i] < e[j] ? i : j;
+      e[up] += need;
+      size[up] = std::ldexp(1.0, e[up]);
     }
+  }
   // the largest absolute sums of a row, over one block and in all, in units
   // of the scales
-  std::vector<double> inv(n);
   for (int i = 0; i < n; ++i) inv[i] = std::ldexp(1.0, -e[i]);
-  double block = 0.0, row = 0.0;
+  double block = 0.0, most = 0.0;
   for (int i = 0; i < n; ++i) {
+    const double* row = S + (size_t)i * n;
     double all = 0.0;
     for (int j0 = 0; j0 < n; j0 += kFxBlock) {
       double s = 0.0;
-      for (int j = j0; j < std::min(n, j0 + kFxBlock); ++j) s += entry(i, j) * inv[i] * inv[j];
-      block = std::max(block, s);
+      for (int j = j0; j < std::min(n, j0 + kFxBlock); ++j) s += std::fabs(row[j]) * inv[j];
+      block = std::max(block, s * inv[i]);
       all += s;
     }
-    row = std::max(row, all);
+    most = std::max(most, all * inv[i]);
   }
   int up = 0;
-  while (up < 16 && (block > (double)kFxBlockSum * (1 << (2 * up)) || row > (double)kFxRowSum * (1 << (2 * up)))) ++up;
+  while (up < 16 && (block > (double)kFxBlockSum * (1 << (2 * up)) || most > (double)kFxRowSum * (1 << (2 * up)))) ++up;
   for (int i = 0; i < n; ++i) e[i] += up;
 }
 
 void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
-                   const std::vector<int32_t>& voff, int threads, std::vector<int64_t>& off, std::vector<int2>& arena,
-                   std::vector<int32_t>& rexp) {
-  const int64_t align = 256 / 8;
+                   const std::vector<int32_t>& voff, int threads, std::vector<int64_t>& off,
+                   std::unique_ptr<int2[]>& arena, int64_t& elems, std::vector<int32_t>& rexp) {
   off.assign(ops.size(), 0);
   int64_t cur = 0, rows = 0;
   for (size_t s = 0; s < ops.size(); ++s) {
-    cur = (cur + align - 1) / align * align;
-    off[s] = cur;
+    off[s] = cur;   // (whole tiles: 8 KB blocks)
     cur += fx_packed_elems(dims[s]);
     rows = std::max<int64_t>(rows, (int64_t)voff[s] + dims[s]);
   }
-  arena.assign((size_t)std::max<int64_t>(cur, 1), make_int2(0, 0));
+  elems = std::max<int64_t>(cur, 1);
+  arena.reset(new int2[elems]);   // (every entry is written below, by the threads)
   rexp.assign((size_t)std::max<int64_t>(rows, 1), 0);
   auto work = [&](int t, int nt) {
+    std::vector<double> S;
     for (size_t s = t; s < ops.size(); s += nt) {
       const int n = dims[s];
-      const std::vector<double>& A = ops[s];
       int32_t* e = &rexp[voff[s]];
       if (n == 0) continue;
-      fx_row_scales(A.data(), n, e);
-      for (int g = 0; g < n; ++g)
-        for (int c = 0; c < (g / kFxTile + 1) * kFxTile && c < n; ++c) {
-          const double v = c == g ? A[(size_t)g * n + g] : 0.5 * (A[(size_t)g * n + c] + A[(size_t)c * n + g]);
-          uint64_t b;
-          std::memcpy(&b, &v, 8);
-          const int64_t q = v == 0.0 ? 0 : fx_quantize(b, kFxBits - e[g] - e[c]);
-          arena[off[s] + fx_entry(g, c)] = make_int2(fx_lo(q), fx_hi(q));
-        }
+      S.resize((size_t)n * n);
+      fx_symmetric_part(ops[s].data(), n, S.data());
+      fx_row_scales(S.data(), n, e);
+      int2* out = arena.get() + off[s];
+      for (int I = 0; I * kFxTile < n; ++I)
+        for (int J = 0; J <= I; ++J)
+          for (int r = 0; r < kFxTile; ++r, out += kFxTile) {
+            const int g = I * kFxTile + r, c0 = J * kFxTile;
+            for (int k = 0; k < kFxTile; ++k) {
+              int64_t q = 0;
+              if (g < n && c0 + k < n) {
+                uint64_t b;
+                std::memcpy(&b, &S[(size_t)g * n + c0 + k], 8);
+                if (b << 1) q = fx_quantize(b, kFxBits - e[g] - e[c0 + k]);
+              }
+              out[((k / 2) ^ (r & 7)) * 2 + k % 2] = make_int2(fx_lo(q), fx_hi(q));   // as fx_entry
+            }
+          }
     }
   };
-  // a thread per million entries or so, not more than asked for
+  // a thread per quarter of a million entries, not more than asked for
   const int nt = (int)std::max<int64_t>(1, std::min<int64_t>(threads, cur >> 18));
   std::vector<std::thread> pool;
   for (int t = 1; t < nt; ++t) pool.emplace_back(work, t, nt);

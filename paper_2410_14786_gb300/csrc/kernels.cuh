@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <memory>
 #include <vector>
 
 #include "internal.hpp"
@@ -38,10 +39,9 @@ cudaError_t launch_sgemv_tma(int precision, const WorkItem* items, int n_items, 
 // the symmetric GEMV above).
 int64_t fx_packed_elems(int n);
 bool fx_gemm_supported(int max_n);
-void fx_row_scales(const double* A, int n, int32_t* e);
 void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
-                   const std::vector<int32_t>& voff, int threads, std::vector<int64_t>& off, std::vector<int2>& arena,
-                   std::vector<int32_t>& rexp);
+                   const std::vector<int32_t>& voff, int threads, std::vector<int64_t>& off,
+                   std::unique_ptr<int2[]>& arena, int64_t& elems, std::vector<int32_t>& rexp);
 // share: the largest operator's part of all operators' entries.
 cudaError_t launch_fx_gemm(const WorkItem* items, int n_items, int max_n, double share, const void* arena,
                            const int32_t* rexp, const double* X, double* Y, const int32_t* yscatter, int nrhs,
