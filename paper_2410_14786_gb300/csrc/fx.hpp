@@ -68,6 +68,18 @@ FX_HD int64_t fx_quantize(uint64_t bits, int add) {
   return (int64_t)(bits >> 63 ? 0 - q : q);
 }
 
+// The same for the words {lo, hi} of a finite x with |x| < 2^E, rounded to
+// `bits` bits and in fewer instructions: round(x 2^(bits - E)), 54 <= bits <= 58.
+// E is at least -1021, so that 0 and subnormal numbers fit too.
+FX_HD int64_t fx_quantize_words(int32_t lo, int32_t hi, int E, int bits = kFxBits) {
+  const int e = (hi >> 20) & 0x7ff;
+  const uint64_t m = ((uint64_t)(uint32_t)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32 | (uint32_t)lo) << (bits - 52);
+  const int d = E - (e ? e : 1) + 1022;   // m < 2^(bits + 1): x 2^(bits - E) = m / 2^(d + 1)
+  const int64_t q = d < 62 ? (int64_t)(((m >> d) + 1) >> 1) : 0;
+  const int64_t s = hi >> 31;
+  return (q ^ s) - s;
+}
+
 FX_HD int32_t fx_hi(int64_t q) { return (int32_t)((q + (1ll << (kFxLow - 1))) >> kFxLow); }
 FX_HD int32_t fx_lo(int64_t q) { return (int32_t)(q - ((int64_t)fx_hi(q) << kFxLow)); }
 
