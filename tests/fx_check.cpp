@@ -53,6 +53,16 @@ int main() {
               "halves of %g", x);
     }
   }
+  // the form from words agrees with the long one
+  for (int i = 0; i < 20000; ++i) {
+    const double x = i < 12 ? special[i] : std::ldexp(nd(g), (int)(g() % 2040) - 1020);
+    if (!std::isfinite(x)) continue;
+    const uint64_t b = bits(x);
+    const int E0 = x == 0.0 ? -1021 : std::max(fx_exponent(b), -1021);
+    for (int E : {E0, E0 + 1, E0 + 7, E0 + 58, E0 + 64, E0 + 2000})
+      for (int nb : {54, 55, kFxBits})
+        REQUIRE(fx_quantize_words((int32_t)b, (int32_t)(b >> 32), E, nb) == fx_quantize(b, nb - E), "words of %g", x);
+  }
   REQUIRE(fx_exponent(bits(INFINITY)) == kFxNonFinite && fx_exponent(bits(-INFINITY)) == kFxNonFinite &&
               fx_exponent(bits(NAN)) == kFxNonFinite, "exponent of a non-finite value");
   // block sums: the extreme halves, and random ones
