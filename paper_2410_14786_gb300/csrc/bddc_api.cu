@@ -444,6 +444,37 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
       CUDA_TRY(upload(h, &h->d_wtx_I[c], tI));
       CUDA_TRY(upload(h, &h->d_wtx_G[c], tG));
     }
+    if (prec == BDDC_PREC_FP32 && h->nrhs_max > 4) {
+      // row tiles and operands of the blocked float32 product
+      auto up_fg = [&](FgOperators& F, const void* arena, const std::vector<int>& dims, const std::vector<int64_t>& off,
+                       const std::vector<int32_t>& ld, const std::vector<int32_t>& voff) -> cudaError_t {
+        std::vector<FgOperand> ops;
+        std::vector<int32_t> xblk(S, 0);
+        F.arena = static_cast<const float*>(arena);
+        for (int s = 0; s < S; ++s) {
+          xblk[s] = (int32_t)F.blocks;
+          if (dims[s]) ops.push_back(FgOperand{voff[s], dims[s], xblk[s]});
+          F.blocks += ld[s] / 4;
+        }
+        F.n_ops = (int)ops.size();
+        cudaError_t e = upload(h, &F.ops, ops);
+        for (int c = 0; c < 3 && e == cudaSuccess; ++c) {
+          const int rt = 32 << c;
+          std::vector<FgItem> it;
+          for (int s = 0; s < S; ++s)
+            for (int r = 0; r < dims[s]; r += rt)
+              it.push_back(FgItem{off[s], ld[s], r, std::min(rt, dims[s] - r), xblk[s], voff[s]});
+          // most work first
+          std::stable_sort(it.begin(), it.end(), [](const FgItem& a, const FgItem& b) { return a.lda > b.lda; });
+          F.n_items[c] = (int)it.size();
+          e = upload(h, &F.items[c], it);
+        }
+        return e;
+      };
+      CUDA_TRY(up_fg(h->fg[0], h->d_aii, dIop, offI, ldI, ioff));
+      CUDA_TRY(up_fg(h->fg[1], h->d_kgg, dG, offG, ldG, goff));
+      CUDA_TRY(dev_alloc(h, &h->d_fgx, fgemm_operand_floats(std::max(h->fg[0].blocks, h->fg[1].blocks), h->nrhs_max)));
+    }
     for (int s = 0; s < S; ++s) {
       opbytes_I += (int64_t)dIop[s] * ldI[s] * elem_bytes(prec);
       opbytes_G += (int64_t)dG[s] * ldG[s] * elem_bytes(prec);
@@ -1308,6 +1339,7 @@ int bddc_autotune(bddc_handle_t h, int32_t nrhs, bddc_tuning_t* out, void* strea
       const bool interior = fam == 0;
       if ((interior ? h->nI_tot : h->nG_tot) == 0) continue;
       if (interior && h->sparse_local) continue;   // the interior solves are sweeps, not a GEMV
+      if (use_fgemm(h, interior, nrhs)) continue;  // not the streamed GEMV
       float best = -1.0f;
       int best_kb = h->tune_stage_kb[fam], best_tc = h->tune_tile_class[fam], best_ns = h->tune_sym_stages[fam];
       auto try_one = [&](int kb, int tc, int ns) {

@@ -826,6 +826,17 @@ bool bgemv_tma_supported(int precision, int max_lda) {
   return kStages * row + xb + 64 <= 200 * 1024;
 }
 
+// Whether a launch for more than 4 columns takes 4 or 8 of them at a time
+// (float32: 16 lanes per row; see dispatch): the launches that bddc_fgemm.cu
+// takes over with the same summation order. (At 4 columns the streamed GEMV is
+// the faster one: 60 against 83 us on 512 operators of 343 rows, 112 against 85
+// at 8 columns, 380 against 218 at 32.)
+bool bgemv_wide(int precision, int max_lda, int nrhs) {
+  if (precision != BDDC_PREC_FP32) return false;
+  const size_t row = ((size_t)max_lda * sizeof(float) + 127) / 128 * 128;
+  return nrhs > 4 && kStages * row + x_bytes<float, 4>(max_lda) + 64 <= 200 * 1024;
+}
+
 int64_t sym_packed_elems(int precision, int n) {
   return precision == BDDC_PREC_FP32 ? tri_off<4>(n) : tri_off<8>(n);
 }

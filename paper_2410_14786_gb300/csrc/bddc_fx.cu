@@ -520,8 +520,8 @@ void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std::vecto
           }
     }
   };
-  // a thread per quarter of a million entries, not more than asked for
-  const int nt = (int)std::max<int64_t>(1, std::min<int64_t>(threads, cur >> 18));
+  // a thread per 65536 entries, not more than asked for
+  const int nt = (int)std::max<int64_t>(1, std::min<int64_t>(threads, cur >> 16));
   std::vector<std::thread> pool;
   for (int t = 1; t < nt; ++t) pool.emplace_back(work, t, nt);
   work(0, nt);

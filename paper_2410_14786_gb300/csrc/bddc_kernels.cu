@@ -597,6 +597,23 @@ cudaError_t interior_sweeps(bddc_handle_s* h, const ApplyWork& W, const double* 
   return launch_scatter_rows(h->nI_tot, nrhs, yscatter, out, Y, st);
 }
 
+}  // namespace
+
+// Whether the blocked float32 product runs an operator family at nrhs columns.
+// Its operand packing is a launch of its own, which small families do not earn
+// back (27 operators of 386 rows, 8 columns: 15.5 against 14 us; 16 of 841: 24
+// against 21.5), while the streamed GEMV loses most where the operand of one
+// operator crowds its shared memory (6 operators of up to 1900 rows, 5 columns:
+// 95 against 26 us).
+bool use_fgemm(const bddc_handle_s* h, bool interior, int nrhs) {
+  const int cols = interior ? h->max_cols_I : h->max_cols_G;
+  if (!h->d_fgx || !h->use_tma || !bgemv_wide(h->precision, cols, nrhs)) return false;
+  const int64_t entries = interior ? h->info.sum_nI2 : h->info.sum_nG2;
+  return cols > 1000 || entries * ((nrhs + 7) / 8) >= 12000000;
+}
+
+namespace {
+
 // One batched application of the interior (A_II^-1) or interface (K_GG)
 // operators of all subdomains.
 // Y = Op X over the interior or interface operators; counts its launches.
@@ -618,6 +635,10 @@ cudaError_t local_op(bddc_handle_s* h, bool interior, const double* X, double* Y
                                        h->d_err, st, h->tune_stage_kb[0], h->tune_sym_stages[0], max_per_sm)
                     : launch_sgemv_tma(h->precision, h->d_wsy_G, h->n_wsy_G, h->max_n_G, h->d_kgg, X, Y, yscatter,
                                        h->d_err, st, h->tune_stage_kb[1], h->tune_sym_stages[1], max_per_sm);
+  }
+  if (use_fgemm(h, interior, nrhs)) {
+    h->launches += h->fg[interior ? 0 : 1].n_ops > 0 ? 2 : 0;
+    return launch_fgemm(h->fg[interior ? 0 : 1], h->d_fgx, X, Y, yscatter, nrhs, st);
   }
   h->launches += (interior ? h->n_wi_I : h->n_wi_G) > 0;
   if (h->use_tma)

@@ -231,6 +231,25 @@ struct TcUnit {
   int32_t kbase;  // first column of the operator in the packed operand buffer
 };
 
+// Float32 operators for blocks of right-hand sides (bddc_fgemm.cu): one row tile
+// of one operator, and one operator's operand (packed in blocks of 4 rows from
+// block xblk on).
+struct FgItem {
+  int64_t moff;
+  int32_t lda, row0, nrows, xblk, yoff;
+};
+struct FgOperand {
+  int32_t xoff, n, xblk;
+};
+struct FgOperators {
+  const float* arena = nullptr;
+  FgItem* items[3] = {nullptr, nullptr, nullptr};   // row tiles of 32, 64 and 128 rows
+  int n_items[3] = {0, 0, 0};
+  FgOperand* ops = nullptr;
+  int n_ops = 0;
+  int64_t blocks = 0;                      // operand blocks of all operators
+};
+
 // One row tile of one dense operator in a batched GEMV launch:
 // Y[yoff + row0 + r] = sum_c Op[row0 + r, c] * X[xoff + c], r < nrows.
 struct WorkItem {
@@ -486,6 +505,9 @@ struct bddc_handle_s {
   int64_t tcB_cols_I = 0, tcB_cols_G = 0;   // sum of padded operator widths
   int tc_maxg_I = 0, tc_maxg_G = 0;          // most row tiles in one unit
   int max_cols_I = 0, max_cols_G = 0;
+  // float32 operators for blocks of right-hand sides: interior, interface; packed operand
+  bddc::FgOperators fg[2];
+  float* d_fgx = nullptr;
   int max_nc = 0;                     // most constraints of one subdomain
   // apply workspace (nrhs_max columns)
   bddc::ApplyWork w;                  // the apply's work vectors (nrhs_max columns)

@@ -53,6 +53,15 @@ cudaError_t launch_bgemv_tma(int precision, const WorkItem* items, int n_items, 
                              const double* X, double* Y, const int32_t* yscatter, int nrhs, int32_t* err,
                              cudaStream_t st, int stage_kb = 12, int max_per_sm = 0);
 
+// Float32 operators times nrhs columns (bddc_fgemm.cu), with the summation order
+// that the streamed GEMV uses where bgemv_wide says so; P: the packed operand,
+// fgemm_operand_floats(blocks, nrhs_max) floats.
+bool bgemv_wide(int precision, int max_lda, int nrhs);
+bool use_fgemm(const bddc_handle_s* h, bool interior, int nrhs);
+size_t fgemm_operand_floats(int64_t blocks, int nrhs_max);
+cudaError_t launch_fgemm(const FgOperators& F, float* P, const double* X, double* Y, const int32_t* yscatter, int nrhs,
+                         cudaStream_t st);
+
 // Tensor-core batched GEMM for blocks of right-hand sides (bddc_tc_gemm.cu).
 // Host packing of dense n x n operators (row-major float64) into the tiled
 // layout; per operator opinfo holds {xoff, n, first packed column, first
