@@ -287,8 +287,8 @@ int bddc_rhs(bddc_handle_t h, const double *f, double *b, int32_t nrhs, void *st
 typedef struct {
     int32_t gemv_stage_kb_interior;   /* streamed-GEMV stage size target, KB, 1..64 (default 12) */
     int32_t gemv_stage_kb_interface;
-    int32_t coarse_rowblock_min_nrhs; /* row-blocked coarse sweeps from this many columns on, 2..65
-                                         (65 = never; default 16) */
+    int32_t coarse_rowblock_min_nrhs; /* row-blocked (matrix-instruction) coarse sweeps from this many columns on, 2..65
+                                         (65 = never; default 2) */
     int32_t gemv_rows_interior;       /* streamed-GEMV work unit: row tile of 64, 128 (default) or 256 rows */
     int32_t gemv_rows_interface;
     int32_t coarse_overlap;           /* 1: the interface operator runs on a second stream, concurrently
@@ -311,7 +311,7 @@ typedef struct {
  * tiles of 64, 128 and 256 rows and stage sizes of 6, 12, 24 and 48 KB of
  * the streamed GEMV of each operator family when the handle uses it, or for
  * the symmetric GEMV 3 or 4 stages of 10 to 24 KB;
- * one-row against four-row coarse sweep units when nrhs >= 2; one launch
+ * one-row against eight-row coarse sweep units when nrhs >= 2; one launch
  * against one launch per level of the one-column coarse sweeps; every split
  * height of the sparse local solver's interior sweeps at one column; whole
  * applies with and without the coarse overlap), apply the fastest and return

@@ -157,225 +157,39 @@ __device__ __forceinline__ double warp_dot_gather(const double* __restrict__ row
   return warp_sum((s0 + s1) + (s2 + s3));
 }
 
-// Several right-hand sides at once: columns k0 .. k0 + nr - 1 (nr <= kNR) of
-// x (row-major, nrhs per row), accumulated into lane-partial sums s[k] with
-// the matrix row read once for all of them.
-constexpr int kNR = 8;
-// Four elements per lane per round (as in warp_dot): out-of-range elements
-// read a valid position and are weighted by zero, so all loads of a round
-// are independent and in flight together.
-__device__ __forceinline__ void warp_dot_multi(const double* __restrict__ row, const double* x, int j0, int j1,
-                                               int nrhs, int k0, int nr, int lane, double (&s)[kNR]) {
-  for (int j = j0 + lane; j < j1; j += 128) {
-    double rv[4];
-    const double* xp[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const bool in = j + 32 * t < j1;
-      rv[t] = in ? __ldg(&row[j + 32 * t]) : 0.0;
-      xp[t] = x + (int64_t)(in ? j + 32 * t : j) * nrhs + k0;
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
-#pragma unroll
-      for (int k = 0; k < kNR; ++k)
-        if (k < nr) s[k] = fma(rv[t], __ldcg(xp[t] + k), s[k]);
-  }
-}
-__device__ __forceinline__ void warp_dot_gather_multi(const double* __restrict__ row, const double* x,
-                                                      const int32_t* __restrict__ idx, int n, int nrhs, int k0,
-                                                      int nr, int lane, double (&s)[kNR]) {
-  for (int j = lane; j < n; j += 128) {
-    double rv[4];
-    int32_t ix[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const bool in = j + 32 * t < n;
-      rv[t] = in ? __ldg(&row[j + 32 * t]) : 0.0;
-      ix[t] = __ldg(&idx[in ? j + 32 * t : j]);
-    }
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const double* xp = x + (int64_t)ix[t] * nrhs + k0;
-#pragma unroll
-      for (int k = 0; k < kNR; ++k)
-        if (k < nr) s[k] = fma(rv[t], __ldcg(xp + k), s[k]);
-    }
-  }
-}
-// Warp sum of the 8 lane-partial sums, left on lanes with (lane & 3) == 0:
-// that lane holds the total of column k = lane >> 2 (three halving
-// exchanges, then two full ones: 9 shuffles instead of 40).
-__device__ __forceinline__ double warp_sum8(double (&s)[kNR], int lane) {
-#pragma unroll
-  for (int o = 16, n = kNR; o >= 4; o >>= 1, n >>= 1) {
-    const bool upper = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < n / 2; ++i) {
-      const double send = upper ? s[i] : s[i + n / 2];
-      const double keep = upper ? s[i + n / 2] : s[i];
-      s[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  double v = s[0];
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  return v;
-}
-
-__device__ void forward_unit(const CoarseArgs& a, const CUnit& w, int lane, int kb, int ke) {
+__device__ void forward_unit(const CoarseArgs& a, const CUnit& w, int lane, int k) {
   const int nrhs = a.nrhs;
   if (w.kind == 0) {
     // y[pos0 + i] = sum_{j <= i} L_PP^-1[i, j] r'[pos0 + j]
     const CNodeDev nd = a.nodes[w.a];
-    const double* row = a.F + nd.foff + (int64_t)w.row * nd.fld;
-    const double* x = a.rp + (int64_t)nd.pos0 * nrhs;
-    double* dst = a.y + (int64_t)(nd.pos0 + w.row) * nrhs;
-    if (ke - kb == 1) {
-      const double s = warp_dot(row, x, 0, w.row + 1, nrhs, kb, lane);
-      if (lane == 0) dst[kb] = s;
-      return;
-    }
-    for (int k0 = kb; k0 < ke; k0 += kNR) {
-      const int nr = min(kNR, nrhs - k0);
-      double s[kNR] = {0, 0, 0, 0, 0, 0, 0, 0};
-      warp_dot_multi(row, x, 0, w.row + 1, nrhs, k0, nr, lane, s);
-      const double v = warp_sum8(s, lane);
-      if ((lane & 3) == 0 && (lane >> 2) < nr) dst[k0 + (lane >> 2)] = v;
-    }
+    const double s = warp_dot(a.F + nd.foff + (int64_t)w.row * nd.fld, a.rp + (int64_t)nd.pos0 * nrhs, 0, w.row + 1,
+                              nrhs, k, lane);
+    if (lane == 0) a.y[(int64_t)(nd.pos0 + w.row) * nrhs + k] = s;
   } else {
     // r'[a] -= sum over the listed contributions, in list order, of
     // M_row . r'_P(node)
     double* dst = &a.rp[(int64_t)w.a * nrhs];
-    if (ke - kb == 1) {
-      double s = 0.0;
-      for (int q = w.b; q < w.e; ++q) {
-        const CContrib c = a.list[q];
-        s += warp_dot(a.F + c.row_off, a.rp + (int64_t)c.x_off * nrhs, 0, c.len, nrhs, kb, lane);
-      }
-      if (lane == 0) dst[kb] = __ldcg(dst + kb) - s;
-      return;
+    double s = 0.0;
+    for (int q = w.b; q < w.e; ++q) {
+      const CContrib c = a.list[q];
+      s += warp_dot(a.F + c.row_off, a.rp + (int64_t)c.x_off * nrhs, 0, c.len, nrhs, k, lane);
     }
-    for (int k0 = kb; k0 < ke; k0 += kNR) {
-      const int nr = min(kNR, nrhs - k0);
-      double s[kNR] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (int q = w.b; q < w.e; ++q) {
-        const CContrib c = a.list[q];
-        warp_dot_multi(a.F + c.row_off, a.rp + (int64_t)c.x_off * nrhs, 0, c.len, nrhs, k0, nr, lane, s);
-      }
-      const double v = warp_sum8(s, lane);
-      if ((lane & 3) == 0 && (lane >> 2) < nr) {
-        double* d = dst + k0 + (lane >> 2);
-        *d = __ldcg(d) - v;
-      }
-    }
+    if (lane == 0) dst[k] = __ldcg(dst + k) - s;
   }
 }
 
-__device__ void backward_unit(const CoarseArgs& a, const CUnit& w, int lane, int kb, int ke) {
+__device__ void backward_unit(const CoarseArgs& a, const CUnit& w, int lane, int k) {
   // u[dof of pos0 + i] = sum_{j >= i} L_PP^-T[i, j] y[pos0 + j] - sum_b M[b, i] u[upd_b]
   const int nrhs = a.nrhs;
   const CNodeDev nd = a.nodes[w.a];
   const double* row = a.B + nd.boff + (int64_t)w.row * nd.bld;
-  const double* yp = a.y + (int64_t)nd.pos0 * nrhs;
-  double* dst = a.u + (int64_t)a.order[nd.pos0 + w.row] * nrhs;
-  if (ke - kb == 1) {
-    const double s = warp_dot(row, yp, w.row, nd.p, nrhs, kb, lane) +
-                     warp_dot_gather(row + nd.p, a.u, a.upd + nd.upd_off, nd.u, nrhs, kb, lane);
-    if (lane == 0) dst[kb] = s;
-    return;
-  }
-  for (int k0 = kb; k0 < ke; k0 += kNR) {
-    const int nr = min(kNR, nrhs - k0);
-    double s[kNR] = {0, 0, 0, 0, 0, 0, 0, 0};
-    warp_dot_multi(row, yp, w.row, nd.p, nrhs, k0, nr, lane, s);
-    warp_dot_gather_multi(row + nd.p, a.u, a.upd + nd.upd_off, nd.u, nrhs, k0, nr, lane, s);
-    const double v = warp_sum8(s, lane);
-    if ((lane & 3) == 0 && (lane >> 2) < nr) dst[k0 + (lane >> 2)] = v;
-  }
+  const double s = warp_dot(row, a.y + (int64_t)nd.pos0 * nrhs, w.row, nd.p, nrhs, k, lane) +
+                   warp_dot_gather(row + nd.p, a.u, a.upd + nd.upd_off, nd.u, nrhs, k, lane);
+  if (lane == 0) a.u[(int64_t)a.order[nd.pos0 + w.row] * nrhs + k] = s;
 }
 
-// Row-blocked sweeps for several right-hand sides: a warp unit covers up to
-// kRB consecutive rows of one node's matrix, so every operand value loaded
-// feeds kRB rows. acc[q][k] += sum_j row_q[j] x[j, k0 + k] for j in [j0, j1);
-// the operand is x[j * nrhs + ...] or, with idx, x[idx[j] * nrhs + ...].
-constexpr int kRB = 4;
-__device__ __forceinline__ void warp_rows_multi(const double* __restrict__ row, int ld, int nq, const double* x,
-                                                const int32_t* __restrict__ idx, int j0, int j1, int nrhs, int k0,
-                                                int nr, int lane, double (&s)[kRB][kNR]) {
-  for (int j = j0 + lane; j < j1; j += 64) {
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int jj = j + 32 * t;
-      const bool in = jj < j1;
-      const int jc = in ? jj : j;
-      double rv[kRB];
-#pragma unroll
-      for (int q = 0; q < kRB; ++q) rv[q] = (in && q < nq) ? __ldg(&row[(int64_t)q * ld + jc]) : 0.0;
-      const int64_t xr = idx ? (int64_t)__ldg(&idx[jc - j0]) : (int64_t)jc;
-      const double* xp = x + xr * nrhs + k0;
-#pragma unroll
-      for (int k = 0; k < kNR; ++k)
-        if (k < nr) {
-          const double xv = __ldcg(xp + k);
-#pragma unroll
-          for (int q = 0; q < kRB; ++q) s[q][k] = fma(rv[q], xv, s[q][k]);
-        }
-    }
-  }
-}
-
-__device__ void forward_rows(const CoarseArgs& a, const CUnit& w, int lane, int kb, int ke) {
-  // y[pos0 + i] = sum_{j <= i} L_PP^-1[i, j] r'[pos0 + j], i in [row, row + b)
-  const int nrhs = a.nrhs, nq = w.b;
-  const CNodeDev nd = a.nodes[w.a];
-  const double* row = a.F + nd.foff + (int64_t)w.row * nd.fld;
-  const double* x = a.rp + (int64_t)nd.pos0 * nrhs;
-  for (int k0 = kb; k0 < ke; k0 += kNR) {
-    const int nr = min(kNR, nrhs - k0);
-    double s[kRB][kNR];
-#pragma unroll
-    for (int q = 0; q < kRB; ++q)
-#pragma unroll
-      for (int k = 0; k < kNR; ++k) s[q][k] = 0.0;
-    warp_rows_multi(row, nd.fld, nq, x, nullptr, 0, w.row + nq, nrhs, k0, nr, lane, s);
-#pragma unroll
-    for (int q = 0; q < kRB; ++q) {
-      const double v = warp_sum8(s[q], lane);
-      if (q < nq && (lane & 3) == 0 && (lane >> 2) < nr)
-        a.y[(int64_t)(nd.pos0 + w.row + q) * nrhs + k0 + (lane >> 2)] = v;
-    }
-  }
-}
-
-__device__ void backward_rows(const CoarseArgs& a, const CUnit& w, int lane, int kb, int ke) {
-  // u[dof of pos0 + i] = sum_{j >= i} L_PP^-T[i, j] y[pos0 + j] - sum_b M[b, i] u[upd_b]
-  const int nrhs = a.nrhs, nq = w.b;
-  const CNodeDev nd = a.nodes[w.a];
-  const double* row = a.B + nd.boff + (int64_t)w.row * nd.bld;
-  const double* yp = a.y + (int64_t)nd.pos0 * nrhs;
-  for (int k0 = kb; k0 < ke; k0 += kNR) {
-    const int nr = min(kNR, nrhs - k0);
-    double s[kRB][kNR];
-#pragma unroll
-    for (int q = 0; q < kRB; ++q)
-#pragma unroll
-      for (int k = 0; k < kNR; ++k) s[q][k] = 0.0;
-    warp_rows_multi(row, nd.bld, nq, yp, nullptr, w.row, nd.p, nrhs, k0, nr, lane, s);
-    warp_rows_multi(row + nd.p, nd.bld, nq, a.u, a.upd + nd.upd_off, 0, nd.u, nrhs, k0, nr, lane, s);
-#pragma unroll
-    for (int q = 0; q < kRB; ++q) {
-      const double v = warp_sum8(s[q], lane);
-      if (q < nq && (lane & 3) == 0 && (lane >> 2) < nr)
-        a.u[(int64_t)a.order[nd.pos0 + w.row + q] * nrhs + k0 + (lane >> 2)] = v;
-    }
-  }
-}
-
-// RB = 1: one row per warp unit (one right-hand side, latency-bound);
-// RB = kRB: row-blocked units (several right-hand sides).
-template <int RB>
-__global__ void __launch_bounds__(RB == 1 ? kThreads : kThreads / 2, 1) k_coarse_solve(CoarseArgs a) {
+// One row and one column per warp unit (few right-hand sides, latency-bound).
+__global__ void __launch_bounds__(kThreads, 1) k_coarse_solve(CoarseArgs a) {
   const int L = a.levels;
   const int32_t* off_f = a.lvl;
   const int32_t* off_b = a.lvl + (L + 1);
@@ -383,12 +197,6 @@ __global__ void __launch_bounds__(RB == 1 ? kThreads : kThreads / 2, 1) k_coarse
   const int lane = threadIdx.x & 31;
   const int gw = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int nw = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
-  // a warp unit is (row unit, block of bw columns): the column blocks of one
-  // unit run on different warps instead of one after the other. One-row
-  // units take one column each (the single-column dot products); the
-  // row-blocked units take kNR columns.
-  const int bw = RB == 1 ? 1 : kNR;
-  const int nrb = (a.nrhs + bw - 1) / bw;
   // r' = r_c in elimination order
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_c * a.nrhs;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -398,26 +206,200 @@ __global__ void __launch_bounds__(RB == 1 ? kThreads : kThreads / 2, 1) k_coarse
   unsigned int epoch = 0;
   if (!grid_sync(a.bar, a.err, epoch, a.bar_extra, a.bar_cycles)) return;
   for (int lv = 0; lv < L; ++lv) {
-    for (int64_t t = (int64_t)off_f[lv] * nrb + gw; t < (int64_t)off_f[lv + 1] * nrb; t += nw) {
-      const int64_t ui = t / nrb;
-      const int kb = (int)(t - ui * nrb) * bw, ke = min(a.nrhs, kb + bw);
-      const CUnit w = a.units[ui];
-      if (RB > 1 && w.kind == 0)
-        forward_rows(a, w, lane, kb, ke);
-      else
-        forward_unit(a, w, lane, kb, ke);
+    for (int64_t t = (int64_t)off_f[lv] * a.nrhs + gw; t < (int64_t)off_f[lv + 1] * a.nrhs; t += nw) {
+      const int64_t ui = t / a.nrhs;
+      forward_unit(a, a.units[ui], lane, (int)(t - ui * a.nrhs));
     }
     if (!grid_sync(a.bar, a.err, epoch, a.bar_extra, a.bar_cycles)) return;
   }
   for (int lv = L - 1; lv >= 0; --lv) {
-    for (int64_t t = (int64_t)off_b[lv] * nrb + gw; t < (int64_t)off_b[lv + 1] * nrb; t += nw) {
-      const int64_t ui = t / nrb;
-      const int kb = (int)(t - ui * nrb) * bw, ke = min(a.nrhs, kb + bw);
-      if (RB > 1)
-        backward_rows(a, a.units[ui], lane, kb, ke);
-      else
-        backward_unit(a, a.units[ui], lane, kb, ke);
+    for (int64_t t = (int64_t)off_b[lv] * a.nrhs + gw; t < (int64_t)off_b[lv + 1] * a.nrhs; t += nw) {
+      const int64_t ui = t / a.nrhs;
+      backward_unit(a, a.units[ui], lane, (int)(t - ui * a.nrhs));
     }
+    if (lv > 0 && !grid_sync(a.bar, a.err, epoch, a.bar_extra, a.bar_cycles)) return;
+  }
+}
+
+// ---- row-blocked sweeps on the float64 matrix instruction (several right-hand sides) ---
+//
+// With several columns the sweeps are dense products of the nodes' matrices with
+// blocks of vectors, and bound by the float64 pipe: 2 FMAs per SM and clock.
+// mma.m8n8k4.f64 (the same IEEE products and sums) runs 7 per SM and clock, so a
+// warp unit here is 8 rows of one node's matrix times 8 columns, four rows of the
+// operand per instruction. A node's M rows form its contribution vector c_t = M
+// r'_P in `cbuf`; before a level runs, the pivots of its nodes collect theirs,
+// r'_P = r_P - sum of the contributions, in node order. That costs a second grid
+// barrier per forward level (about 2 us) and makes every product a plain one.
+// Measured against one row and column per warp (k_coarse_solve): 2863 coarse dofs,
+// 2 columns 118 us both, 8 columns 116 against 187, 64 columns 341 against 763;
+// interior forest of 160000 dofs, 4 columns: 0.55 against 2.54 ms. (4 rows x 8
+// columns per warp on the float64 pipe, the form before: 376 us for 32 columns on
+// 1011 coarse dofs, now 126.) What is left is latency: barriers and one or two
+// rounds of loads per level.
+struct MmaArgs {
+  const CNodeDev* nodes;
+  const MUnit* units;
+  const int32_t* upd;        // update-set dofs
+  const int32_t* order;      // position -> dof
+  const int32_t* lvl;        // offsets: units [L + 1 forward][L + 1 backward], pivots of a level [L + 1]
+  const int32_t* piv;        // positions of the pivots, by level
+  const int32_t* cptr;       // [n + 1] contributions of a position: entries cidx of cbuf
+  const int32_t* cidx;
+  const double* F;
+  const double* B;
+  const double* r;           // dof order
+  double* rp;                // r' (positions)
+  double* y;                 // y (positions)
+  double* u;                 // solution (dof order)
+  double* cbuf;
+  unsigned int* bar;
+  int32_t* err;
+  int levels, nrhs;
+  unsigned int bar_extra;
+  long long bar_cycles;
+};
+
+__device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+               : "+d"(c[0]), "+d"(c[1])
+               : "d"(a), "d"(b));
+}
+
+// c += rows 0 .. nrow - 1 of m, columns [j0, j1), times the operand rows: row j is
+// that of the position xa + j for j < p (of the dof ord[j] where ord is given), and
+// that of the dof idx[j - p] of xb from p on. Lane l holds entry (l / 4, 4 s + l % 4)
+// of the matrix and operand entry (4 s + l % 4, col) for the steps s; 4 steps are
+// loaded before they are used. What lies outside is 0 (col = -1: the whole column).
+__device__ __forceinline__ void mma_rows(double (&c)[2], const double* __restrict__ m, int64_t ld, int nrow,
+                                         const double* xa, const int32_t* __restrict__ ord, int p, const double* xb,
+                                         const int32_t* __restrict__ idx, int j0, int j1, int nrhs, int col, int lane) {
+  const int r = lane >> 2, kk = lane & 3;
+  const double* mr = m + (int64_t)(r < nrow ? r : 0) * ld;
+  for (int j = j0 + kk; j - kk < j1; j += 16) {
+    double av[4], bv[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const int jj = j + 4 * s;
+      const bool in = jj < j1;
+      av[s] = in && r < nrow ? __ldg(mr + jj) : 0.0;
+      bv[s] = 0.0;
+      if (in && col >= 0) {
+        const double* x = jj < p ? xa + (int64_t)(ord ? __ldg(ord + jj) : jj) * nrhs : xb + (int64_t)__ldg(idx + (jj - p)) * nrhs;
+        bv[s] = __ldcg(x + col);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) dmma(c, av[s], bv[s]);
+  }
+}
+
+// One unit and column block: the whole product (parts = 1) or part `part` of its
+// columns, in multiples of 16.
+__device__ __forceinline__ void mma_unit(const MmaArgs& a, const MUnit& w, const CNodeDev& nd, int nrow, bool leaves,
+                                         int k0, int lane, int part, int parts, double (&c)[2]) {
+  const int col = k0 + (lane >> 2) < a.nrhs ? k0 + (lane >> 2) : -1;
+  int j0 = w.kind == 2 ? w.row : 0, j1 = w.kind == 0 ? w.row + nrow : w.kind == 1 ? nd.p : nd.p + nd.u;
+  if (parts > 1) {
+    const int chunk = ((j1 - j0 + parts - 1) / parts + 15) / 16 * 16;
+    j0 += part * chunk;
+    j1 = min(j1, j0 + chunk);
+  }
+  if (w.kind == 2)
+    mma_rows(c, a.B + nd.boff + (int64_t)w.row * nd.bld, nd.bld, nrow, a.y + (int64_t)nd.pos0 * a.nrhs, nullptr, nd.p,
+             a.u, a.upd + nd.upd_off, j0, j1, a.nrhs, col, lane);
+  else   // (the leaves' r' is r itself)
+    mma_rows(c, a.F + nd.foff + (int64_t)(w.kind ? nd.p + w.row : w.row) * nd.fld, nd.fld, nrow,
+             leaves ? a.r : a.rp + (int64_t)nd.pos0 * a.nrhs, leaves ? a.order + nd.pos0 : nullptr, nd.p, nullptr,
+             nullptr, j0, j1, a.nrhs, col, lane);
+}
+
+// Entries (lane / 4, 2 (lane % 4) + {0, 1}) of the unit's result.
+__device__ __forceinline__ void mma_store(const MmaArgs& a, const MUnit& w, const CNodeDev& nd, int nrow, int k0,
+                                          int lane, const double (&c)[2]) {
+  const int r = lane >> 2, k = k0 + 2 * (lane & 3);
+  if (r >= nrow) return;
+  double* out = w.kind == 0   ? a.y + (int64_t)(nd.pos0 + w.row + r) * a.nrhs
+                : w.kind == 1 ? a.cbuf + (int64_t)(nd.upd_off + w.row + r) * a.nrhs
+                              : a.u + (int64_t)a.order[nd.pos0 + w.row + r] * a.nrhs;
+  if (k < a.nrhs) out[k] = c[0];
+  if (k + 1 < a.nrhs) out[k + 1] = c[1];
+}
+
+// The units [u0, u1) of one level, times ncb column blocks. Many of them: one per
+// warp. Few (the top levels, whose rows are long): one per block, the warps sharing
+// its columns and the partial sums added in warp order; one warp alone is limited
+// to its quarter of the SM's pipe (the top levels took two thirds of 304 us).
+constexpr int kMmaWarps = kThreads / 64;
+__device__ __forceinline__ void mma_level(const MmaArgs& a, int u0, int u1, int ncb, bool leaves, double (*red)[64],
+                                          int& buf) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int warps = blockDim.x >> 5;
+  const int64_t total = (int64_t)(u1 - u0) * ncb;
+  if (total >= 8 * (int64_t)gridDim.x) {
+    // consecutive units on different SMs
+    for (int64_t t = (int64_t)warp * gridDim.x + blockIdx.x; t < total; t += (int64_t)gridDim.x * warps) {
+      const MUnit w = a.units[u0 + t / ncb];
+      const int k0 = (int)(t % ncb) * 8;
+      const CNodeDev nd = a.nodes[w.node];
+      const int nrow = min(8, (w.kind == 1 ? nd.u : nd.p) - w.row);
+      double c[2] = {0.0, 0.0};
+      mma_unit(a, w, nd, nrow, leaves, k0, lane, 0, 1, c);
+      mma_store(a, w, nd, nrow, k0, lane, c);
+    }
+    return;
+  }
+  for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+    const MUnit w = a.units[u0 + t / ncb];
+    const int k0 = (int)(t % ncb) * 8;
+    const CNodeDev nd = a.nodes[w.node];
+    const int nrow = min(8, (w.kind == 1 ? nd.u : nd.p) - w.row);
+    double c[2] = {0.0, 0.0};
+    mma_unit(a, w, nd, nrow, leaves, k0, lane, warp, warps, c);
+    double(*rb)[64] = red + buf * kMmaWarps;
+    rb[warp][2 * lane] = c[0];
+    rb[warp][2 * lane + 1] = c[1];
+    __syncthreads();   // (the other buffer's reader passed the barrier before)
+    if (warp == 0) {
+      c[0] = c[1] = 0.0;
+      for (int q = 0; q < warps; ++q) {
+        c[0] += rb[q][2 * lane];
+        c[1] += rb[q][2 * lane + 1];
+      }
+      mma_store(a, w, nd, nrow, k0, lane, c);
+    }
+    buf ^= 1;
+  }
+}
+
+__global__ void __launch_bounds__(kThreads / 2, 1) k_sweeps_mma(MmaArgs a) {
+  __shared__ double red[2 * kMmaWarps][64];
+  int buf = 0;
+  const int L = a.levels, nrhs = a.nrhs, ncb = (nrhs + 7) / 8;
+  const int32_t* off_f = a.lvl;
+  const int32_t* off_b = a.lvl + (L + 1);
+  const int32_t* off_p = a.lvl + 2 * (L + 1);
+  unsigned int epoch = 0;
+  for (int lv = 0; lv < L; ++lv) {
+    if (lv > 0) {
+      // r' at the pivots of this level
+      const int64_t np = (int64_t)(off_p[lv + 1] - off_p[lv]) * nrhs;
+      for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t q = i / nrhs;
+        const int k = (int)(i - q * nrhs), pos = a.piv[off_p[lv] + q];
+        double s = 0.0;
+        const int e1 = a.cptr[pos + 1];
+#pragma unroll 4
+        for (int e = a.cptr[pos]; e < e1; ++e) s += __ldcg(&a.cbuf[(int64_t)a.cidx[e] * nrhs + k]);
+        a.rp[(int64_t)pos * nrhs + k] = __ldg(&a.r[(int64_t)a.order[pos] * nrhs + k]) - s;
+      }
+      if (!grid_sync(a.bar, a.err, epoch, a.bar_extra, a.bar_cycles)) return;
+    }
+    mma_level(a, off_f[lv], off_f[lv + 1], ncb, lv == 0, red, buf);
+    if (!grid_sync(a.bar, a.err, epoch, a.bar_extra, a.bar_cycles)) return;
+  }
+  for (int lv = L - 1; lv >= 0; --lv) {
+    mma_level(a, off_b[lv], off_b[lv + 1], ncb, false, red, buf);
     if (lv > 0 && !grid_sync(a.bar, a.err, epoch, a.bar_extra, a.bar_cycles)) return;
   }
 }
@@ -1203,13 +1185,13 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
   std::vector<int32_t> pos(cf.n);
   for (int64_t i = 0; i < cf.n; ++i) pos[cf.order[i]] = (int32_t)i;
   // warp units: forward levels (L_PP^-1 rows, then one unit per receiving
-  // position with its (node, M row) pairs in node order), then backward
-  // levels; rows of kinds 0 and 2 in blocks of rb (1, or kRB for the
-  // multi-RHS sweeps). The contribution list is the same for both blockings.
+  // position with its (node, M row) pairs in node order), then backward levels
   std::vector<CContrib> list;
   std::vector<std::vector<int32_t>> contrib(cf.n);
   std::vector<int32_t> touched;
-  auto make_units = [&](int rb, std::vector<CUnit>& units, std::vector<int32_t>& lvl, bool fill_list) {
+  std::vector<CUnit> units;
+  std::vector<int32_t> lvl;
+  {
     lvl.assign(2 * (L + 1) + 1, 0);
     int32_t lcur = 0;
     for (int lv = 0; lv < L; ++lv) {
@@ -1218,7 +1200,7 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
       for (int t = 0; t < nn; ++t) {
         const CoarseNode& T = cf.nodes[t];
         if (T.height != lv || T.p == 0) continue;
-        for (int i = 0; i < T.p; i += rb) units.push_back(CUnit{0, t, i, std::min(rb, T.p - i), 0});
+        for (int i = 0; i < T.p; ++i) units.push_back(CUnit{0, t, i, 1, 0});
         for (int b = 0; b < T.u; ++b) {
           const int32_t w = pos[T.upd[b]];
           if (contrib[w].empty()) touched.push_back(w);
@@ -1231,7 +1213,7 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
         const int32_t b0 = lcur;
         for (size_t q = 0; q < contrib[w].size(); q += 2) {
           const CNodeDev& nd = nodes[contrib[w][q]];
-          if (fill_list) list.push_back(CContrib{nd.foff + (int64_t)(nd.p + contrib[w][q + 1]) * nd.fld, nd.pos0, nd.p, 0});
+          list.push_back(CContrib{nd.foff + (int64_t)(nd.p + contrib[w][q + 1]) * nd.fld, nd.pos0, nd.p, 0});
           ++lcur;
         }
         units.push_back(CUnit{1, w, 0, b0, lcur});
@@ -1244,16 +1226,54 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
       for (int t = 0; t < nn; ++t) {
         const CoarseNode& T = cf.nodes[t];
         if (T.height != lv || T.p == 0) continue;
-        for (int i = 0; i < T.p; i += rb) units.push_back(CUnit{2, t, i, std::min(rb, T.p - i), 0});
+        for (int i = 0; i < T.p; ++i) units.push_back(CUnit{2, t, i, 1, 0});
       }
     }
     lvl[(L + 1) + L] = (int)units.size();
     lvl[2 * (L + 1)] = (int32_t)cf.n;
-  };
-  std::vector<CUnit> units, units4;
-  std::vector<int32_t> lvl, lvl4;
-  make_units(1, units, lvl, true);
-  make_units(kRB, units4, lvl4, false);
+  }
+  // the row-blocked form: 8-row units per level (longest rows first), the
+  // pivots of a level, and for every position the entries of the contribution
+  // buffer (update-set numbering) that it collects, in node order
+  std::vector<MUnit> munits;
+  std::vector<int32_t> mlvl(3 * (L + 1), 0), piv, cptr(cf.n + 1, 0), cidx;
+  if (multi) {
+    auto by_length = [&](size_t from, auto len) {
+      std::stable_sort(munits.begin() + from, munits.end(),
+                       [&](const MUnit& x, const MUnit& y) { return len(x) > len(y); });
+    };
+    for (int lv = 0; lv < L; ++lv) {
+      mlvl[lv] = (int)munits.size();
+      mlvl[2 * (L + 1) + lv] = (int)piv.size();
+      for (int t = 0; t < nn; ++t) {
+        const CoarseNode& T = cf.nodes[t];
+        if (T.height != lv || T.p == 0) continue;
+        for (int i = 0; i < T.p; i += 8) munits.push_back(MUnit{t, i, 0});
+        for (int i = 0; i < T.u; i += 8) munits.push_back(MUnit{t, i, 1});
+        for (int i = 0; i < T.p; ++i) piv.push_back(nodes[t].pos0 + i);
+      }
+      by_length(mlvl[lv], [&](const MUnit& x) { return x.kind ? nodes[x.node].p : x.row + 8; });
+    }
+    mlvl[L] = (int)munits.size();
+    mlvl[2 * (L + 1) + L] = (int)piv.size();
+    for (int lv = 0; lv < L; ++lv) {
+      mlvl[(L + 1) + lv] = (int)munits.size();
+      for (int t = 0; t < nn; ++t)
+        if (cf.nodes[t].height == lv)
+          for (int i = 0; i < cf.nodes[t].p; i += 8) munits.push_back(MUnit{t, i, 2});
+      by_length(mlvl[(L + 1) + lv], [&](const MUnit& x) { return nodes[x.node].p + nodes[x.node].u - x.row; });
+    }
+    mlvl[(L + 1) + L] = (int)munits.size();
+    for (int t = 0; t < nn; ++t)
+      if (cf.nodes[t].p)
+        for (int b = 0; b < cf.nodes[t].u; ++b) cptr[pos[cf.nodes[t].upd[b]] + 1]++;
+    for (int64_t i = 0; i < cf.n; ++i) cptr[i + 1] += cptr[i];
+    cidx.resize(cptr[cf.n]);
+    std::vector<int32_t> fill(cptr.begin(), cptr.end() - 1);
+    for (int t = 0; t < nn; ++t)
+      if (cf.nodes[t].p)
+        for (int b = 0; b < cf.nodes[t].u; ++b) cidx[fill[pos[cf.nodes[t].upd[b]]]++] = nodes[t].upd_off + b;
+  }
   if ((e = up(h, &S.F, F)) != cudaSuccess) return e;
   std::vector<double>().swap(F);
   if ((e = up(h, &S.B, B)) != cudaSuccess) return e;
@@ -1261,21 +1281,29 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
   if (!multi) return cudaSuccess;
   if ((e = up(h, &S.nodes, nodes)) != cudaSuccess) return e;
   if ((e = up(h, &S.units, units)) != cudaSuccess) return e;
-  if ((e = up(h, &S.units4, units4)) != cudaSuccess) return e;
-  if ((e = up(h, &S.lvl4, lvl4)) != cudaSuccess) return e;
+  if ((e = up(h, &S.munits, munits)) != cudaSuccess) return e;
+  if ((e = up(h, &S.mlvl, mlvl)) != cudaSuccess) return e;
+  if ((e = up(h, &S.piv, piv)) != cudaSuccess) return e;
+  if ((e = up(h, &S.cptr, cptr)) != cudaSuccess) return e;
+  if ((e = up(h, &S.cidx, cidx)) != cudaSuccess) return e;
+  {
+    void* cb = nullptr;
+    if ((e = cudaMalloc(&cb, std::max<size_t>(1, upd.size()) * h->nrhs_max * sizeof(double))) != cudaSuccess) return e;
+    h->allocations.push_back(cb);
+    S.mcbuf = static_cast<double*>(cb);
+  }
   if ((e = up(h, &S.list, list)) != cudaSuccess) return e;
   if ((e = up(h, &S.upd, upd)) != cudaSuccess) return e;
   if ((e = up(h, &S.order, cf.order)) != cudaSuccess) return e;
   if ((e = up(h, &S.lvl, lvl)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_solve<1>, kThreads, 0)) != cudaSuccess)
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_solve, kThreads, 0)) != cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorNotSupported;
   S.grid = sms * std::min(per_sm, 2);
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_solve<kRB>, kThreads / 2, 0)) !=
-      cudaSuccess)
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweeps_mma, kThreads / 2, 0)) != cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorNotSupported;
-  S.grid4 = sms * std::min(per_sm, 2);
+  S.mgrid = sms * std::min(per_sm, 2);
   return cudaSuccess;
 }
 
@@ -1417,22 +1445,25 @@ cudaError_t launch_sweeps(bddc_handle_s* h, const SweepSet& S, const double* r, 
     h->launches++;
     return e;
   }
-  // row blocking pays from about 16 right-hand sides on (fewer, longer units
-  // per level; measured on 10439 coarse dofs); the autotuner may move the
-  // threshold
-  const bool blocked = nrhs > 1 && nrhs >= h->tune_coarse_rb_min;
-  CoarseArgs a{S.nodes, blocked ? S.units4 : S.units, S.list, S.upd, S.order, blocked ? S.lvl4 : S.lvl,
-               S.F, S.B, r, rp, y, u, S.bar, h->d_err, S.levels, nrhs, extra, cycles};
+  // the row-blocked form from tune_coarse_rb_min right-hand sides on (the
+  // autotuner may move the threshold)
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(narrow ? h->c_sms : blocked ? S.grid4 : S.grid);
-  cfg.blockDim = dim3((narrow || blocked) ? kThreads / 2 : kThreads);
-  cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = blocked ? cudaLaunchKernelEx(&cfg, k_coarse_solve<kRB>, a) : cudaLaunchKernelEx(&cfg, k_coarse_solve<1>, a);
   h->launches++;
-  return e;
+  if (nrhs >= h->tune_coarse_rb_min) {
+    MmaArgs m{S.nodes, S.munits, S.upd, S.order, S.mlvl, S.piv, S.cptr, S.cidx, S.F, S.B, r, rp, y, u, S.mcbuf, S.bar,
+              h->d_err, S.levels, nrhs, extra, cycles};
+    cfg.gridDim = dim3(narrow ? h->c_sms : S.mgrid);
+    cfg.blockDim = dim3(kThreads / 2);
+    return cudaLaunchKernelEx(&cfg, k_sweeps_mma, m);
+  }
+  CoarseArgs a{S.nodes, S.units, S.list, S.upd, S.order, S.lvl, S.F, S.B, r, rp, y, u, S.bar, h->d_err, S.levels, nrhs,
+               extra, cycles};
+  cfg.gridDim = dim3(narrow ? h->c_sms : S.grid);
+  cfg.blockDim = dim3(narrow ? kThreads / 2 : kThreads);
+  return cudaLaunchKernelEx(&cfg, k_coarse_solve, a);
 }
 
 }  // namespace bddc

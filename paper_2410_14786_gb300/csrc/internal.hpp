@@ -22,10 +22,14 @@ struct CNodeDev {
 // One warp's unit of a coarse-sweep level: kind 0 = row `row` of L_PP^-1 of
 // node `a` (forward), kind 1 = all contributions to the dof at elimination
 // position `a` from this level (contributions [b, e)), kind 2 = row `row` of
-// the backward matrix of node `a`. In the row-blocked lists (several
-// right-hand sides) kinds 0 and 2 cover rows [row, row + b).
+// the backward matrix of node `a`.
 struct CUnit {
   int32_t kind, a, row, b, e;
+};
+// One warp's unit of the row-blocked sweeps: 8 rows from `row` on of node
+// `node`: kind 0 of L_PP^-1, 1 of M, 2 of the backward matrix.
+struct MUnit {
+  int32_t node, row, kind;
 };
 // One output value of a coarse sweep in the gather form (one right-hand
 // side): value = sum_{j < len} C[off + j] * X[I[off + j]], where an index
@@ -100,12 +104,15 @@ struct SweepSet {
   double* B = nullptr;          // backward matrices [L_PP^-T , -M^T]
   CNodeDev* nodes = nullptr;
   CUnit* units = nullptr;       // warp units, forward levels then backward levels
-  CUnit* units4 = nullptr;      // the same with kinds 0 and 2 blocked by 4 rows
   CContrib* list = nullptr;     // contributions of the receiving units
   int32_t* upd = nullptr;       // update-set dofs of every node
   int32_t* order = nullptr;     // elimination position -> dof
   int32_t* lvl = nullptr;       // unit offsets: [L+1 forward][L+1 backward], then n
-  int32_t* lvl4 = nullptr;
+  // row-blocked form (several right-hand sides): units, level offsets, pivots by
+  // level, contributions per position, contribution buffer (nrhs_max columns)
+  MUnit* munits = nullptr;
+  int32_t *mlvl = nullptr, *piv = nullptr, *cptr = nullptr, *cidx = nullptr;
+  double* mcbuf = nullptr;
   double* gC = nullptr;
   float* gC32 = nullptr;        // the gather form's coefficients in float32 (per-level form only), else null
   float* x32 = nullptr;         // with gC32: float32 copies of r', y and r (n each), the operands the sweeps read
@@ -114,7 +121,7 @@ struct SweepSet {
   int32_t* gwo[2] = {nullptr, nullptr};   // [phases][warps + 1]
   unsigned int* bar = nullptr;
   int64_t n = 0;                // dofs
-  int levels = 0, grid = 0, grid4 = 0, g_blocks = 0;
+  int levels = 0, grid = 0, mgrid = 0, g_blocks = 0;
   int g_fwd = 0, g_phases = 0;  // gather form: forward-type phases, all phases
   int64_t nnz = 0;              // stored entries of F and B
   int64_t g_entries = 0;        // stored entries of the gather form
@@ -412,7 +419,7 @@ struct bddc_handle_s {
   int tune_stage_kb[2] = {12, 12};   // streamed GEMV stage size: interior, interface operators
   int tune_sym_stages[2] = {4, 4};   // stages of the symmetric GEMV: interior, interface operators
   int tune_tile_class[2] = {1, 1};   // streamed GEMV row tile 64 << class: interior, interface
-  int tune_coarse_rb_min = 16;       // row-blocked coarse sweeps from this many right-hand sides on
+  int tune_coarse_rb_min = 2;       // row-blocked coarse sweeps from this many right-hand sides on
   int tune_overlap = 0;              // interface operator concurrent with the coarse residual and solve
   // second stream of the apply and its fork / join events, one set per
   // capture sequence: [0] direct launches and the solve graph's prologue,
