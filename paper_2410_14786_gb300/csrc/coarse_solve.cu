@@ -224,19 +224,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_solve(CoarseArgs a) {
 // ---- row-blocked sweeps on the float64 matrix instruction (several right-hand sides) ---
 //
 // With several columns the sweeps are dense products of the nodes' matrices with
-// blocks of vectors, and bound by the float64 pipe: 2 FMAs per SM and clock.
-// mma.m8n8k4.f64 (the same IEEE products and sums) runs 7 per SM and clock, so a
-// warp unit here is 8 rows of one node's matrix times 8 columns, four rows of the
-// operand per instruction. A node's M rows form its contribution vector c_t = M
-// r'_P in `cbuf`; before a level runs, the pivots of its nodes collect theirs,
-// r'_P = r_P - sum of the contributions, in node order. That costs a second grid
-// barrier per forward level (about 2 us) and makes every product a plain one.
+// blocks of vectors. What bounded them was not the float64 pipe but latency: a row
+// and a column (or 4 rows and 8 columns) per warp, with their loads, reductions and
+// chains of contributions one after another. A unit here is 8 rows of one node's
+// matrix times 8 columns on mma.m8n8k4.f64: the instruction runs at the float64
+// pipe's rate (measured 1.8 FMAs per SM and clock), but one load of a matrix entry
+// serves 8 columns, one of an operand entry 8 rows, and nothing is reduced across
+// lanes. A node's M rows form its contribution vector c_t = M r'_P in `cbuf`;
+// before a level runs, the pivots of its nodes collect theirs, r'_P = r_P - sum of
+// the contributions, in node order. That costs a second grid barrier per forward
+// level (about 2 us) and makes every product a plain one.
 // Measured against one row and column per warp (k_coarse_solve): 2863 coarse dofs,
 // 2 columns 118 us both, 8 columns 116 against 187, 64 columns 341 against 763;
 // interior forest of 160000 dofs, 4 columns: 0.55 against 2.54 ms. (4 rows x 8
-// columns per warp on the float64 pipe, the form before: 376 us for 32 columns on
-// 1011 coarse dofs, now 126.) What is left is latency: barriers and one or two
-// rounds of loads per level.
+// columns per warp with float64 FMAs, the form before: 376 us for 32 columns on
+// 1011 coarse dofs, now 126.) What is left at 8 columns is latency: barriers and
+// one or two rounds of loads per level (the pipe is 23 % busy).
 struct MmaArgs {
   const CNodeDev* nodes;
   const MUnit* units;
@@ -328,8 +331,8 @@ __device__ __forceinline__ void mma_store(const MmaArgs& a, const MUnit& w, cons
 
 // The units [u0, u1) of one level, times ncb column blocks. Many of them: one per
 // warp. Few (the top levels, whose rows are long): one per block, the warps sharing
-// its columns and the partial sums added in warp order; one warp alone is limited
-// to its quarter of the SM's pipe (the top levels took two thirds of 304 us).
+// its columns and the partial sums added in warp order: one warp alone is limited
+// to its quarter of the SM's pipe (with warps alone the 2863 dofs took 304 us).
 constexpr int kMmaWarps = kThreads / 64;
 __device__ __forceinline__ void mma_level(const MmaArgs& a, int u0, int u1, int ncb, bool leaves, double (*red)[64],
                                           int& buf) {
