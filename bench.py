@@ -366,8 +366,8 @@ def run_gb300(args):
     op_bytes = (2 * inf["interior_op_bytes"] + inf["interface_op_bytes"]
                 + 8 * 2 * nrhs * (2 * inf["n_interior"] + inf["n_interface_copies"]))
     achieved = op_bytes / (op_ms * 1e-3) / 1e9
-    kname = ("k_tc_gemm" if inf["tensor_cores"] else "k_sgemv_tma" if inf["symmetric_operators"]
-             else "k_bgemv_tma")
+    kname = ("k_tc_gemm" if inf["tensor_cores"] else "k_bgemv_tma" if not inf["symmetric_operators"]
+             else "k_fx_gemm" if headline == "fp64" else "k_sgemv_tma")
     wl = WORKLOAD if args.config == 2 and nrhs == 1 else p.name
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": MEASURED_TRAFFIC.get((wl, headline, kname)), "peak_kind": peak_kind,
