@@ -155,12 +155,15 @@ typedef struct {
                               most); 0 = one per SM. Fewer blocks give each warp more
                               units of every level (for small coarse problems). >= 0 */
     int32_t full_operators; /* 1: store the symmetric local operators in full. 0 (default):
-                              in the FP32 and BF16 forms on the CUDA cores with
-                              nrhs_max = 1, and in the FP64 form (as 58-bit block fixed
-                              point, unless an operator has about 3900 rows or more),
-                              A_II^-1 and K_GG are stored as their lower
-                              triangles (about half the bytes) and applied by the
-                              symmetric streamed kernels; elsewhere in full */
+                              A_II^-1 and K_GG are stored as their lower triangles in
+                              the FP32 and BF16 forms on the CUDA cores with nrhs_max = 1
+                              (about half the bytes, applied by the symmetric streamed
+                              GEMV), and in the FP64 form up to 3968 rows, in block fixed
+                              point with the float64 triangles beside it (together about
+                              the bytes of the full operators). A row of a product is
+                              used in fixed point where it is as accurate as the float64
+                              sum relative to its own sum |a_ij| |x_j|, and summed in
+                              float64 elsewhere. Elsewhere in full */
     int32_t history;       /* PCG iterations whose scalars (||r_k||, alpha_k, beta_k) the
                               handle keeps for bddc_pcg_history, 0..100000; 0 = none */
     int32_t coarse_cg_maxit; /* BDDC_COARSE_CG: iteration limit of the coarse CG, >= 0;
@@ -183,7 +186,7 @@ typedef struct {
     int64_t coarse_bytes;               /* device bytes of the coarse operator */
     int64_t device_bytes;               /* all device memory the handle holds */
     int64_t apply_bytes_1rhs;           /* algorithmic HBM bytes of one apply, nrhs = 1 */
-    int64_t interior_op_bytes;          /* bytes of all A_II^-1 blocks as stored */
+    int64_t interior_op_bytes;          /* bytes of all A_II^-1 blocks, as one product reads them */
     int64_t interface_op_bytes;         /* bytes of all K_GG blocks as stored */
     int64_t n_interface_copies;         /* sum over subdomains of interface nodes */
     int64_t kernel_launches;            /* kernels launched by this handle so far */

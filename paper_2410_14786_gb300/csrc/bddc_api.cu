@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/bddc.h"
+#include "fx_pack.hpp"
 #include "internal.hpp"
 #include "kernels.cuh"
 
@@ -198,6 +199,24 @@ std::vector<WorkItem> make_items(const std::vector<int64_t>& off, const std::vec
   return items;
 }
 
+// Whole operators, largest first.
+std::vector<WorkItem> make_whole_items(const std::vector<int64_t>& off, const std::vector<int>& dims,
+                                       const std::vector<int32_t>& voff, int eb) {
+  std::vector<WorkItem> items;
+  for (size_t s = 0; s < dims.size(); ++s)
+    if (dims[s]) items.push_back(WorkItem{off[s], padded_ld(dims[s], eb), dims[s], 0, dims[s], voff[s], voff[s]});
+  std::stable_sort(items.begin(), items.end(),
+                   [](const WorkItem& a, const WorkItem& b) { return a.ncols > b.ncols; });
+  return items;
+}
+
+// Whether a family of float64 operators runs in block fixed point.
+bool use_fx_family(const std::vector<int>& dims, int nrhs_max) {
+  int n = 0;
+  for (int d : dims) n = std::max(n, d);
+  return n > 0 && fx_gemm_supported(n);
+}
+
 int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
   const int S = hs.n_sub;
   int64_t in_coarse_bytes = 0, coarse_read_1rhs = 0;
@@ -325,8 +344,8 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
     return upload(h, reinterpret_cast<__nv_bfloat16**>(dst), a);
   };
   int64_t opbytes_I = 0, opbytes_G = 0;
-  const int max_dim = std::max(dIop.empty() ? 0 : *std::max_element(dIop.begin(), dIop.end()),
-                               dG.empty() ? 0 : *std::max_element(dG.begin(), dG.end()));
+  auto largest = [](const std::vector<int>& d) { return d.empty() ? 0 : *std::max_element(d.begin(), d.end()); };
+  const int max_dim = std::max(largest(dIop), largest(dG));
   if (h->use_tc) {
     // tensor-core path: operators in the MMA tile layout, no row-major copy
     auto up_tc = [&](auto tag, const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
@@ -369,25 +388,15 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
     h->allocations.push_back(pB);
     h->d_tcB = pB;
     h->use_tma = false;
-  } else if (!h->full_operators && (prec == BDDC_PREC_FP64 ? fx_gemm_supported(max_dim)
-                                                           : h->nrhs_max == 1 && sgemv_tma_supported(prec, max_dim))) {
-    // symmetric operators (float32 and bfloat16: one right-hand side): lower
-    // triangles, one work item per operator (largest first)
+  } else if (!h->full_operators && prec != BDDC_PREC_FP64 && h->nrhs_max == 1 && sgemv_tma_supported(prec, max_dim)) {
+    // symmetric operators, one right-hand side: lower triangles, one work item
+    // per operator (largest first)
     auto up_sym = [&](const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
                       const std::vector<int32_t>& voff, void** arena, WorkItem** items, int* n_items, int* max_n,
-                      int64_t* bytes, int32_t** rexp) -> cudaError_t {
+                      int64_t* bytes) -> cudaError_t {
       std::vector<int64_t> off;
       cudaError_t e;
-      if (prec == BDDC_PREC_FP64) {
-        std::unique_ptr<int2[]> a;
-        int64_t elems = 0;
-        std::vector<int32_t> re;
-        fx_pack_lower(ops, dims, voff, hs.threads, off, a, elems, re);
-        arena_bytes += elems * sizeof(int2);
-        e = dev_alloc(h, reinterpret_cast<int2**>(arena), elems);
-        if (e == cudaSuccess) e = cudaMemcpy(*arena, a.get(), elems * sizeof(int2), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = upload(h, rexp, re);
-      } else if (prec == BDDC_PREC_FP32) {
+      if (prec == BDDC_PREC_FP32) {
         auto a = pack_lower<float>(ops, dims, prec, off, cvt_f);
         arena_bytes += a.size() * sizeof(float);
         e = upload(h, reinterpret_cast<float**>(arena), a);
@@ -397,33 +406,83 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
         e = upload(h, reinterpret_cast<__nv_bfloat16**>(arena), a);
       }
       if (e != cudaSuccess) return e;
-      std::vector<WorkItem> it;
+      std::vector<WorkItem> it = make_whole_items(off, dims, voff, elem_bytes(prec));
       *bytes = 0;
-      *max_n = 0;
-      for (size_t s = 0; s < dims.size(); ++s) {
-        if (dims[s] == 0) continue;
-        it.push_back(WorkItem{off[s], padded_ld(dims[s], elem_bytes(prec)), dims[s], 0, dims[s], voff[s], voff[s]});
-        *bytes += (prec == BDDC_PREC_FP64 ? fx_packed_elems(dims[s]) : sym_packed_elems(prec, dims[s])) * elem_bytes(prec);
-        *max_n = std::max(*max_n, dims[s]);
-      }
-      std::stable_sort(it.begin(), it.end(), [](const WorkItem& a, const WorkItem& b) { return a.ncols > b.ncols; });
+      for (int n : dims) *bytes += sym_packed_elems(prec, n) * elem_bytes(prec);
+      *max_n = largest(dims);
       *n_items = (int)it.size();
       return upload(h, items, it);
     };
     CUDA_TRY(up_sym(hs.AIIinv, dIop, ioff, reinterpret_cast<void**>(&h->d_aii), &h->d_wsy_I, &h->n_wsy_I,
-                    &h->max_n_I, &opbytes_I, &h->d_rexp_I));
+                    &h->max_n_I, &opbytes_I));
     CUDA_TRY(up_sym(hs.Kgg, dG, goff, reinterpret_cast<void**>(&h->d_kgg), &h->d_wsy_G, &h->n_wsy_G, &h->max_n_G,
-                    &opbytes_G, &h->d_rexp_G));
-    h->use_fx = prec == BDDC_PREC_FP64;
-    if (opbytes_I) h->fx_share[0] = 8.0 * fx_packed_elems(h->max_n_I) / opbytes_I;
-    if (opbytes_G) h->fx_share[1] = 8.0 * fx_packed_elems(h->max_n_G) / opbytes_G;
-    h->use_sym = h->use_tma = !h->use_fx;
+                    &opbytes_G));
+    h->use_sym = h->use_tma = true;
   } else {
-    CUDA_TRY(up_arena(hs.AIIinv, dIop, offI, ldI, &h->d_aii));
-    CUDA_TRY(up_arena(hs.Kgg, dG, offG, ldG, &h->d_kgg));
+    // float64: the families that run in block fixed point, as lower triangles of
+    // tiles (one work item per operator, largest first); what follows then lists
+    // no operators of theirs
+    auto up_fx = [&](int fam, const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
+                     const std::vector<int32_t>& voff, const std::vector<uint8_t>& drop, WorkItem** items, int* n_items,
+                     int* max_n, int64_t* bytes) -> cudaError_t {
+      FxPacked pk;
+      fx_pack_lower(ops, dims, voff, drop, hs.threads, pk);
+      int32_t *halves = nullptr, *rexp = nullptr;
+      double* values = nullptr;
+      int8_t* shift = nullptr;
+      cudaError_t e = dev_alloc(h, &halves, 2 * pk.elems);
+      if (e == cudaSuccess) e = cudaMemcpy(halves, pk.halves.get(), 8 * pk.elems, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = dev_alloc(h, &values, pk.elems);
+      if (e == cudaSuccess) e = cudaMemcpy(values, pk.values.get(), 8 * pk.elems, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess) e = upload(h, &rexp, pk.rexp);
+      if (e == cudaSuccess) e = upload(h, &shift, pk.shift);
+      if (e != cudaSuccess) return e;
+      arena_bytes += 16 * pk.elems;
+      h->fx[fam] = FxForm{halves, values, rexp, shift};
+      h->use_fx[fam] = true;
+      const std::vector<WorkItem> it = make_whole_items(pk.off, dims, voff, 8);
+      // (the float64 tiles are read for single rows only)
+      *bytes = 0;
+      for (int n : dims) *bytes += 8 * fx_packed_elems(n);
+      *max_n = largest(dims);
+      h->fx_share[fam] = 8.0 * fx_packed_elems(*max_n) / *bytes;
+      *n_items = (int)it.size();
+      return upload(h, items, it);
+    };
+    std::vector<int> dIf = dIop, dGf = dG;   // the operators kept in full
+    if (prec == BDDC_PREC_FP64 && !h->full_operators) {
+      const bool fx_I = use_fx_family(dIop, h->nrhs_max), fx_G = use_fx_family(dG, h->nrhs_max);
+      int64_t elems = 0;
+      for (int s = 0; s < S; ++s) elems += (fx_I ? fx_packed_elems(dIop[s]) : 0) + (fx_G ? fx_packed_elems(dG[s]) : 0);
+      // both forms of the tiles take about what the full operators take, but up to
+      // several times that where operators are smaller than a tile: not where
+      // they would take more than half of the device's free memory
+      size_t free_bytes = 0, all_bytes = 0;
+      CUDA_TRY(cudaMemGetInfo(&free_bytes, &all_bytes));
+      const bool fits = 16 * elems <= (int64_t)(free_bytes / 2);
+      if (fx_I && fits) {
+        CUDA_TRY(up_fx(0, hs.AIIinv, dIop, ioff, {}, &h->d_wsy_I, &h->n_wsy_I, &h->max_n_I, &opbytes_I));
+        dIf.assign(S, 0);
+      }
+      if (fx_G && fits) {
+        // K_GG's rows of nodes that are a constraint by themselves are zero in
+        // exact arithmetic, rounding noise as computed: packed as zeros
+        std::vector<uint8_t> drop(h->nG_tot, 0);
+        for (int s = 0; s < S; ++s)
+          for (int32_t g : hs.sub_globs[s])
+            if (hs.glob_nodes[g].size() == 1) {
+              const auto& G = hs.sub_G[s];
+              drop[goff[s] + (std::lower_bound(G.begin(), G.end(), hs.glob_nodes[g][0]) - G.begin())] = 1;
+            }
+        CUDA_TRY(up_fx(1, hs.Kgg, dG, goff, drop, &h->d_wsy_G, &h->n_wsy_G, &h->max_n_G, &opbytes_G));
+        dGf.assign(S, 0);
+      }
+    }
+    CUDA_TRY(up_arena(hs.AIIinv, dIf, offI, ldI, &h->d_aii));
+    CUDA_TRY(up_arena(hs.Kgg, dGf, offG, ldG, &h->d_kgg));
     const int tile = 64;
-    auto itI = make_items(offI, ldI, dIop, ioff, tile);
-    auto itG = make_items(offG, ldG, dG, goff, tile);
+    auto itI = make_items(offI, ldI, dIf, ioff, tile);
+    auto itG = make_items(offG, ldG, dGf, goff, tile);
     h->n_wi_I = (int)itI.size();
     h->n_wi_G = (int)itG.size();
     h->max_cols_I = ldI.empty() ? 0 : *std::max_element(ldI.begin(), ldI.end());
@@ -435,8 +494,8 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
     // (the autotuner picks one per operator family; 128 by default)
     for (int c = 0; c < 3; ++c) {
       const int ttile = 64 << c;
-      auto tI = make_items(offI, ldI, dIop, ioff, ttile);
-      auto tG = make_items(offG, ldG, dG, goff, ttile);
+      auto tI = make_items(offI, ldI, dIf, ioff, ttile);
+      auto tG = make_items(offG, ldG, dGf, goff, ttile);
       h->n_wtx_I[c] = (int)tI.size();
       h->n_wtx_G[c] = (int)tG.size();
       if (!items_aligned(tI, elem_bytes(prec)) || !items_aligned(tG, elem_bytes(prec)))
@@ -476,8 +535,8 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
       CUDA_TRY(dev_alloc(h, &h->d_fgx, fgemm_operand_floats(std::max(h->fg[0].blocks, h->fg[1].blocks), h->nrhs_max)));
     }
     for (int s = 0; s < S; ++s) {
-      opbytes_I += (int64_t)dIop[s] * ldI[s] * elem_bytes(prec);
-      opbytes_G += (int64_t)dG[s] * ldG[s] * elem_bytes(prec);
+      opbytes_I += (int64_t)dIf[s] * ldI[s] * elem_bytes(prec);
+      opbytes_G += (int64_t)dGf[s] * ldG[s] * elem_bytes(prec);
     }
   }
   h->coarse_dense = hs.coarse_dense;
@@ -673,7 +732,7 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
   in.interior_factor_entries = ifac_entries;
   in.interface_op_bytes = opbytes_G;
   in.tensor_cores = h->use_tc ? 1 : 0;
-  in.symmetric_operators = h->use_sym || h->use_fx ? 1 : 0;
+  in.symmetric_operators = h->use_sym || h->use_fx[0] || h->use_fx[1] ? 1 : 0;
   in.n_interface_copies = h->nG_tot;
   in.coarse_factor_entries = h->c_nnz;
   in.coarse_update_total = h->cs.update_total;
@@ -1339,7 +1398,7 @@ int bddc_autotune(bddc_handle_t h, int32_t nrhs, bddc_tuning_t* out, void* strea
       const bool interior = fam == 0;
       if ((interior ? h->nI_tot : h->nG_tot) == 0) continue;
       if (interior && h->sparse_local) continue;   // the interior solves are sweeps, not a GEMV
-      if (use_fgemm(h, interior, nrhs)) continue;  // not the streamed GEMV
+      if (h->use_fx[fam] || use_fgemm(h, interior, nrhs)) continue;  // not the streamed GEMV
       float best = -1.0f;
       int best_kb = h->tune_stage_kb[fam], best_tc = h->tune_tile_class[fam], best_ns = h->tune_sym_stages[fam];
       auto try_one = [&](int kb, int tc, int ns) {

@@ -623,12 +623,12 @@ cudaError_t local_op(bddc_handle_s* h, bool interior, const double* X, double* Y
                      cudaStream_t st, int max_per_sm = 0) {
   if (interior && h->sparse_local) return interior_sweeps(h, h->w, X, Y, yscatter, nrhs, st);
   if (h->use_tc) return launch_tc_gemm(h, interior, X, Y, yscatter, nrhs, st);
-  if (h->use_fx) {
-    h->launches += (interior ? h->n_wsy_I : h->n_wsy_G) > 0;
-    return interior ? launch_fx_gemm(h->d_wsy_I, h->n_wsy_I, h->max_n_I, h->fx_share[0], h->d_aii, h->d_rexp_I, X, Y,
-                                     yscatter, nrhs, h->d_err, st)
-                    : launch_fx_gemm(h->d_wsy_G, h->n_wsy_G, h->max_n_G, h->fx_share[1], h->d_kgg, h->d_rexp_G, X, Y,
-                                     yscatter, nrhs, h->d_err, st);
+  const int fam = interior ? 0 : 1;
+  if (h->use_fx[fam]) {
+    h->launches += 1;
+    return launch_fx_gemm(interior ? h->d_wsy_I : h->d_wsy_G, interior ? h->n_wsy_I : h->n_wsy_G,
+                          interior ? h->max_n_I : h->max_n_G, h->fx_share[fam], h->fx[fam], X, Y, yscatter, nrhs, h->d_err,
+                          st);
   }
   if (h->use_sym) {
     if (nrhs != 1) return cudaErrorInvalidValue;   // nrhs_max is 1 on this path

@@ -257,6 +257,14 @@ struct FgOperators {
   int64_t blocks = 0;                      // operand blocks of all operators
 };
 
+// Float64 operators of one family in block fixed point (fx_pack.hpp), on the device.
+struct FxForm {
+  const int32_t* halves = nullptr;   // fixed-point tiles
+  const double* values = nullptr;    // the same tiles in float64
+  const int32_t* rexp = nullptr;     // row exponents (compact interior / interface numbering)
+  const int8_t* shift = nullptr;     // tile shifts
+};
+
 // One row tile of one dense operator in a batched GEMV launch:
 // Y[yoff + row0 + r] = sum_c Op[row0 + r, c] * X[xoff + c], r < nrows.
 struct WorkItem {
@@ -492,14 +500,12 @@ struct bddc_handle_s {
   bool use_tma = false;
   // symmetric operators as packed lower triangles (one work item per operator)
   bool use_sym = false;
-  bool use_fx = false;                // float64: the same in block fixed point (any number of columns)
+  bool use_fx[2] = {false, false};    // float64 in block fixed point (any number of columns): interior, interface
   bool full_operators = false;        // option: keep them in full
   bddc::WorkItem* d_wsy_I = nullptr; int n_wsy_I = 0;
   bddc::WorkItem* d_wsy_G = nullptr; int n_wsy_G = 0;
   int max_n_I = 0, max_n_G = 0;
-  // float64: entries in block fixed point, with the exponent of every row
-  // (compact interior / interface numbering)
-  int32_t *d_rexp_I = nullptr, *d_rexp_G = nullptr;
+  bddc::FxForm fx[2];                 // the fixed-point operators: interior, interface
   double fx_share[2] = {0, 0};        // the largest operator's part of all entries: interior, interface
   // tensor-core path: tiled arenas (d_aii / d_kgg then hold the tiled layout)
   bool use_tc = false;

@@ -5,7 +5,6 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <memory>
 #include <vector>
 
 #include "internal.hpp"
@@ -32,20 +31,13 @@ bool sgemv_tma_supported(int precision, int max_n);
 cudaError_t launch_sgemv_tma(int precision, const WorkItem* items, int n_items, int max_n, const void* arena,
                              const double* X, double* Y, const int32_t* yscatter, int32_t* err, cudaStream_t st,
                              int stage_kb, int n_stages, int max_per_sm = 0);
-// The float64 operators in block fixed point (bddc_fx.cu, fx.hpp), lower
-// triangles of tiles: entries of one n x n operator, whether the kernel
-// supports the size, the host packing (entries, and the exponent of every
-// row at voff[s] + row), and Y = Op X for nrhs columns (work items as for
-// the symmetric GEMV above).
-int64_t fx_packed_elems(int n);
+// The float64 operators in block fixed point (bddc_fx.cu), packed by fx_pack.hpp:
+// whether the kernel supports the size, and Y = Op X for nrhs columns (work items
+// as for the symmetric GEMV above; share: the largest operator's part of all
+// operators' entries).
 bool fx_gemm_supported(int max_n);
-void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std::vector<int>& dims,
-                   const std::vector<int32_t>& voff, int threads, std::vector<int64_t>& off,
-                   std::unique_ptr<int2[]>& arena, int64_t& elems, std::vector<int32_t>& rexp);
-// share: the largest operator's part of all operators' entries.
-cudaError_t launch_fx_gemm(const WorkItem* items, int n_items, int max_n, double share, const void* arena,
-                           const int32_t* rexp, const double* X, double* Y, const int32_t* yscatter, int nrhs,
-                           int32_t* err, cudaStream_t st);
+cudaError_t launch_fx_gemm(const WorkItem* items, int n_items, int max_n, double share, const FxForm& A, const double* X,
+                           double* Y, const int32_t* yscatter, int nrhs, int32_t* err, cudaStream_t st);
 // stage_kb: target bytes of one shared-memory stage, in KB (1..64; 12 by default,
 // the autotuner may choose another per operator family); max_per_sm > 0 caps
 // the blocks per SM (to leave room for a concurrent kernel).
