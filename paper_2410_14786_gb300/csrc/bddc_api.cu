@@ -210,11 +210,25 @@ std::vector<WorkItem> make_whole_items(const std::vector<int64_t>& off, const st
   return items;
 }
 
-// Whether a family of float64 operators runs in block fixed point.
+// Whether a family of float64 operators runs in block fixed point. A unit of that
+// kernel is a whole operator, at the cost of three block barriers and a chain of
+// loads (about 3 us), which many small operators don't earn back against the
+// streamed GEMV's row tiles: at one column 4096 operators of 27 rows take 124 us
+// against 21, 1728 of 64 rows 59 against 23, of 125 rows 67 against 67, of 136 rows
+// 68 against 106; more columns favour fixed point earlier (4096 operators of 89
+// rows: 129 against 83 us at one column, 166 against 160 at 2, 254 against 397 at
+// 4; 576 of 49 rows 56 against 48 at 8, of 81 rows 60 against 105). Up to about 32
+// operators either form is one wave of launch latency.
 bool use_fx_family(const std::vector<int>& dims, int nrhs_max) {
-  int n = 0;
-  for (int d : dims) n = std::max(n, d);
-  return n > 0 && fx_gemm_supported(n);
+  int n = 0, count = 0;
+  double sq = 0.0;
+  for (int d : dims) {
+    n = std::max(n, d);
+    count += d > 0;
+    sq += (double)d * d;
+  }
+  const double least = nrhs_max == 1 ? 125.0 : nrhs_max < 4 ? 100.0 : nrhs_max < 8 ? 80.0 : 70.0;
+  return n > 0 && fx_gemm_supported(n) && (count <= 32 || sq >= least * least * count);
 }
 
 int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
