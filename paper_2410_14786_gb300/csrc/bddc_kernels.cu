@@ -20,7 +20,7 @@
 #include <algorithm>
 #include <cstdint>
 
-#include "fx.hpp"
+#include "elem_grad.hpp"
 #include "kernels.cuh"
 
 namespace bddc {
@@ -429,55 +429,11 @@ __global__ void __launch_bounds__(kThreads) k_mass(int ne, int nrhs, double scal
   }
 }
 
-// Adjoint gradient, element term: g[e] = - sum_k lambda_k,e^T K_ref u_k,e. K_ref
-// of the Q1 element depends only on the number of coordinate bits in which two
-// local nodes differ, and its rows sum to 0, so with weights w = -K_ref[a][b]
-//   lambda^T K_ref u = sum over node pairs of w (lambda_a - lambda_b) (u_a - u_b).
-// 3D: w = h / 12 for the pairs two or three bits apart (face and cube diagonals)
-// and 0 along the edges, so the pairs lie within the two tetrahedra of even and of
-// odd corners, plus the four cube diagonals (a, 7 - a) between them:
-//   sum = sum_a lambda_a (5 u_a - u_(7 - a)) - S_even T_even - S_odd T_odd
-// with T, S the sums of u and lambda over a tetrahedron.
-// In float64 its pipe is the bound (72 operations per element and column for the
-// matrix as it stands, 53 us on 72^3 elements; 32 in this form, 29 us, but with three
-// times the error). So the 3D form runs in block fixed point (fx.hpp), the values of
-// one element and column rounded to 55 bits of their largest: the sums are then
-// exact, and no cancellation between them costs accuracy: 23 us.
-
-// a b in units of 2^(2 kEgLow), as (h, m): h + m 2^-kEgLow (low halves' product dropped).
-constexpr int kEgBits = 55, kEgLow = 28;
-__device__ __forceinline__ void eg_mac(int64_t& h, int64_t& m, int64_t a, int64_t b) {
-  const int ah = (int)((a + (1ll << (kEgLow - 1))) >> kEgLow), bh = (int)((b + (1ll << (kEgLow - 1))) >> kEgLow);
-  const int al = (int)a - (ah << kEgLow), bl = (int)b - (bh << kEgLow);
-  h += (int64_t)ah * bh;
-  m += (int64_t)ah * bl;
-  m += (int64_t)al * bh;
-}
-// sum over the pairs of one element, times 2^-(Eu + El)
-__device__ double eg_fixed(const double (&uv)[8], const double (&lv)[8], int Eu, int El) {
-  int64_t u[8], l[8];
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    u[a] = fx_quantize_words(__double2loint(uv[a]), __double2hiint(uv[a]), Eu, kEgBits);
-    l[a] = fx_quantize_words(__double2loint(lv[a]), __double2hiint(lv[a]), El, kEgBits);
-  }
-  int64_t h = 0, m = 0;
-#pragma unroll
-  for (int a = 0; a < 8; ++a) eg_mac(h, m, 5 * u[a] - u[7 - a], l[a]);
-  eg_mac(h, m, -(u[0] + u[3] + u[5] + u[6]), l[0] + l[3] + l[5] + l[6]);
-  eg_mac(h, m, -(u[7] + u[4] + u[2] + u[1]), l[7] + l[4] + l[2] + l[1]);
-  h += m >> kEgLow;
-  m &= (1ll << kEgLow) - 1;
-  return fma((double)m, 1.0 / (double)(1 << kEgLow), (double)h);
-}
-// Largest exponent (of 0 and subnormal numbers: -1021) of 8 values; above 1024: not all finite.
-__device__ __forceinline__ int eg_exponent(const double (&v)[8]) {
-  int e = 1;
-#pragma unroll
-  for (int a = 0; a < 8; ++a) e = max(e, (__double2hiint(v[a]) >> 20) & 0x7ff);
-  return e - 1022;
-}
-
+// Adjoint gradient, element term: g[e] = - sum_k lambda_k,e^T K_ref u_k,e, one
+// thread per element. 3D: block fixed point where it is as accurate as the float64
+// products, those elsewhere (elem_grad.hpp). What bounds the float64 form is its
+// pipe: 72 operations per element and column, 53 us on 72^3 elements; the integer
+// form takes 22.6 us. 2D: the sum over the node pairs.
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_elem_grad(int ne, int nrhs, double c1, double c2,
                                                         const double* __restrict__ u, const double* __restrict__ lam,
@@ -506,19 +462,11 @@ __global__ void __launch_bounds__(kThreads) k_elem_grad(int ne, int nrhs, double
       if constexpr (DIM == 3) {
         const int Eu = eg_exponent(uv), El = eg_exponent(lv);
         const int k2 = Eu + El + 2 * (kEgLow - kEgBits);
-        if (Eu > 1024 || El > 1024) {   // an infinity or NaN: the float64 products
-          const double coef[4] = {-4.0 * c2, 0.0, c2, c2};
-#pragma unroll
-          for (int a = 0; a < 8; ++a) {
-            double t = 0.0;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) t = fma(coef[__popc(a ^ b)], uv[b], t);
-            s = fma(lv[a], t, s);
-          }
-        } else {
-          const double v = eg_fixed(uv, lv, Eu, El);
+        double v;
+        if (Eu > 1024 || El > 1024 || !eg_fixed(uv, lv, Eu, El, v))   // (not all finite, or not accurate)
+          s = eg_products(uv, lv, c2, s);
+        else
           s = k2 > -900 && k2 < 900 ? fma(-c2 * __hiloint2double((k2 + 1023) << 20, 0), v, s) : s - c2 * scalbn(v, k2);
-        }
       } else {
         // the four edges and the two diagonals
         auto pair = [&](int a, int b) { return (lv[a] - lv[b]) * (uv[a] - uv[b]); };
