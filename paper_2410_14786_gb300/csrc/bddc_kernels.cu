@@ -373,8 +373,8 @@ __global__ void k_zero_nodes(int64_t n, int nrhs, const int32_t* __restrict__ no
 // matrix-free Q1 operators on the structured grid
 // ---------------------------------------------------------------------------
 // b = M f on the free nodes. The Q1 mass matrix is the tensor product of the 1D
-// ones, h / 6 [1 4 1], so a row of 27 (9) products is three (two) passes of one
-// add and one FMA. What bounds it is the float64 pipe, so the passes share their
+// ones, h / 6 [1 4 1], so a row of 27 (9) products is three (two) passes of two or
+// three operations. What bounds it is the float64 pipe, so the passes share their
 // work: thread (i, y) of a block marches along z; per plane it forms its own row
 // sum along x, the rows exchange theirs through shared memory for the sum along
 // y, and the last three planes' sums give a node: about 8 float64 operations per
@@ -397,11 +397,12 @@ __global__ void __launch_bounds__(kThreads) k_mass(int ne, int nrhs, double scal
   // 3D: blockIdx.y rows, blockIdx.z steps; 2D: every row of threads marches by itself
   const int y = DIM == 3 ? blockIdx.y * kMassRows + ty : 0;
   const int z0 = DIM == 3 ? blockIdx.z * kMassSteps : (blockIdx.y * kMassRows + ty) * kMassSteps;
-  // 1 4 1 along x at row yy of step z (0 where nothing depends on it)
+  // 1 4 1 along x at row yy of step z, times scale (here, so that no sum overflows
+  // that its result does not); 0 where nothing depends on it
   auto row_sum = [&](int yy, int z) {
     if (!inner || z < 0 || z > ne || yy < 0 || yy > ne) return 0.0;
     const double* p = f + z * plane + (DIM == 3 ? yy * w : 0) + i;
-    return fma(4.0, __ldg(p), __ldg(p - nrhs) + __ldg(p + nrhs));
+    return fma(4.0 * scale, __ldg(p), fma(scale, __ldg(p - nrhs), scale * __ldg(p + nrhs)));
   };
   const bool row_free = DIM == 2 || (y > 0 && y < ne);
   double s0 = 0.0, s1 = 0.0;                                  // sums of the two planes before
@@ -421,7 +422,7 @@ __global__ void __launch_bounds__(kThreads) k_mass(int ne, int nrhs, double scal
     }
     const int zo = z - 1;   // the plane that is complete now
     if (q >= 2 && i < w && zo <= ne && (DIM == 2 || y <= ne)) {
-      const double v = inner && row_free && zo > 0 && zo < ne ? scale * fma(4.0, s1, s0 + s2) : 0.0;
+      const double v = inner && row_free && zo > 0 && zo < ne ? fma(4.0, s1, s0 + s2) : 0.0;
       b[zo * plane + (DIM == 3 ? y * w : 0) + i] = v;
     }
     s0 = s1;
