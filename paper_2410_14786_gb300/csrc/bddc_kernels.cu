@@ -464,15 +464,23 @@ __global__ void __launch_bounds__(kThreads) k_elem_grad(int ne, int nrhs, double
         const int Eu = eg_exponent(uv), El = eg_exponent(lv);
         const int k2 = Eu + El + 2 * (kEgLow - kEgBits);
         double v;
-        if (Eu > 1024 || El > 1024 || !eg_fixed(uv, lv, Eu, El, v))   // (not all finite, or not accurate)
-          s = eg_products(uv, lv, c2, s);
-        else
-          s = k2 > -900 && k2 < 900 ? fma(-c2 * __hiloint2double((k2 + 1023) << 20, 0), v, s) : s - c2 * scalbn(v, k2);
+        if (Eu > 1024 || El > 1024 || !eg_fixed(uv, lv, Eu, El, v)) {   // (not all finite, or not accurate)
+          const double coef[4] = {-4.0 * c2, 0.0, c2, c2};
+          s = eg_products(uv, lv, coef, s);
+        } else {
+          s = k2 > -900 && k2 < 900 ? fma(-c2 * __hiloint2double((k2 + 1023) << 20, 0), v, s) : s + scalbn(-c2 * v, k2);
+        }
       } else {
-        // the four edges and the two diagonals
-        auto pair = [&](int a, int b) { return (lv[a] - lv[b]) * (uv[a] - uv[b]); };
-        s = fma(-c1, (pair(0, 1) + pair(2, 3)) + (pair(0, 2) + pair(1, 3)), s);
-        s = fma(-c2, pair(0, 3) + pair(1, 2), s);
+        const int Eu = eg_exponent(uv), El = eg_exponent(lv);
+        if (max(max(Eu, El), Eu + El) > 1000) {   // differences or their products might overflow (or are not finite)
+          const double coef[4] = {-2.0 * c1 - c2, c1, c2, 0.0};
+          s = eg_products(uv, lv, coef, s);
+        } else {
+          // the four edges and the two diagonals
+          auto pair = [&](int a, int b) { return (lv[a] - lv[b]) * (uv[a] - uv[b]); };
+          s = fma(-c1, (pair(0, 1) + pair(2, 3)) + (pair(0, 2) + pair(1, 3)), s);
+          s = fma(-c2, pair(0, 3) + pair(1, 2), s);
+        }
       }
     }
     g[e] = -s;

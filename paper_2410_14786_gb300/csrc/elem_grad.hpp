@@ -43,10 +43,11 @@ FX_HD uint64_t eg_bits(double v) {
 #endif
 }
 
-// Largest exponent (of 0 and subnormal numbers: -1021) of 8 values; above 1024: not all finite.
-FX_HD int eg_exponent(const double (&v)[8]) {
+// Largest exponent (of 0 and subnormal numbers: -1021) of N values; above 1024: not all finite.
+template <int N>
+FX_HD int eg_exponent(const double (&v)[N]) {
   int e = 1;
-  for (int a = 0; a < 8; ++a) {
+  for (int a = 0; a < N; ++a) {
     const int x = (int)(eg_bits(v[a]) >> 52) & 0x7ff;
     e = x > e ? x : e;
   }
@@ -92,18 +93,19 @@ FX_HD bool eg_fixed(const double (&uv)[8], const double (&lv)[8], int Eu, int El
   return (uint64_t)T[0] * S[0] + (uint64_t)T[1] * S[1] >= 1ull << (2 * (kEgBits - 32) - kEgCertBits);
 }
 
-// s + lambda^T K_ref u by the float64 products, c2 = -w.
-FX_HD double eg_products(const double (&u)[8], const double (&l)[8], double c2, double s) {
-  const double coef[4] = {-4.0 * c2, 0.0, c2, c2};
+// s + lambda^T K_ref u by the float64 products, coef[d] the entry of K_ref between
+// nodes d bits apart.
+template <int N>
+FX_HD double eg_products(const double (&u)[N], const double (&l)[N], const double (&coef)[4], double s) {
 #if defined(__CUDACC__)
 #pragma unroll
 #endif
-  for (int a = 0; a < 8; ++a) {
+  for (int a = 0; a < N; ++a) {
     double t = 0.0;
 #if defined(__CUDACC__)
 #pragma unroll
 #endif
-    for (int b = 0; b < 8; ++b) {
+    for (int b = 0; b < N; ++b) {
       const int d = a ^ b, bits = (d & 1) + ((d >> 1) & 1) + (d >> 2);
       t = fma(coef[bits], u[b], t);
     }

@@ -25,6 +25,7 @@ int main() {
       const double h = 1.0 / (1 + g() % 200), c2 = -h / 12, su = std::pow(10.0, 4 * nd(g)), sl = std::pow(10.0, 4 * nd(g));
       const int peak = (int)(g() % 8), axis = 1 << (g() % 3);
       double u[8], l[8];
+      const double coef[4] = {-4.0 * c2, 0.0, c2, c2};
       for (int a = 0; a < 8; ++a) {
         if (kind == 0) u[a] = su * (1 + 0.1 * nd(g)), l[a] = sl * (1 + 0.1 * nd(g));
         if (kind == 1) u[a] = nd(g), l[a] = nd(g);
@@ -48,7 +49,7 @@ int main() {
       const int Eu = eg_exponent(u), El = eg_exponent(l);
       double v;
       const bool holds = eg_fixed(u, l, Eu, El, v);
-      worst64 = std::fmax(worst64, (double)(std::fabs(eg_products(u, l, c2, 0.0) - exact) / size));
+      worst64 = std::fmax(worst64, (double)(std::fabs(eg_products(u, l, coef, 0.0) - exact) / size));
       if (holds) {
         ++taken;
         worst = std::fmax(worst, (double)(std::fabs(-c2 * std::ldexp(v, Eu + El + 2 * (kEgLow - kEgBits)) - exact) / size));
