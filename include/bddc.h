@@ -292,7 +292,8 @@ typedef struct {
     int32_t gemv_stage_kb_interior;   /* streamed-GEMV stage size target, KB, 1..64 (default 12) */
     int32_t gemv_stage_kb_interface;
     int32_t coarse_rowblock_min_nrhs; /* row-blocked (matrix-instruction) coarse sweeps from this many columns on, 2..65
-                                         (65 = never; default 2) */
+                                         (65 = never; default 2, or 4 for coarse factors of more than 5e6
+                                         entries; the sparse local solver's sweeps are always row-blocked) */
     int32_t gemv_rows_interior;       /* streamed-GEMV work unit: row tile of 64, 128 (default) or 256 rows */
     int32_t gemv_rows_interface;
     int32_t coarse_overlap;           /* 1: the interface operator runs on a second stream, concurrently

@@ -1322,7 +1322,7 @@ int bddc_clear_device_error(bddc_handle_t h) {
 
 int bddc_get_tuning(bddc_handle_t h, bddc_tuning_t* out) {
   if (!h || !out) return fail(BDDC_ERR_INVALID_ARG, "null handle or output");
-  *out = bddc_tuning_t{h->tune_stage_kb[0], h->tune_stage_kb[1], h->tune_coarse_rb_min,
+  *out = bddc_tuning_t{h->tune_stage_kb[0], h->tune_stage_kb[1], h->cs.rb_min,
                        64 << h->tune_tile_class[0], 64 << h->tune_tile_class[1], h->tune_overlap,
                        h->tune_sym_stages[0], h->tune_sym_stages[1], h->is.block_min_height,
                        h->cs.use_level ? 1 : 0};
@@ -1355,7 +1355,7 @@ int bddc_set_tuning(bddc_handle_t h, const bddc_tuning_t* in) {
   h->tune_stage_kb[1] = in->gemv_stage_kb_interface;
   h->tune_sym_stages[0] = in->sym_stages_interior;
   h->tune_sym_stages[1] = in->sym_stages_interface;
-  h->tune_coarse_rb_min = in->coarse_rowblock_min_nrhs;
+  h->cs.rb_min = in->coarse_rowblock_min_nrhs;
   h->cs.use_level = in->coarse_level_launches == 1 && !h->cs.lv.empty();
   if (h->is.block_form) {
     // the interior sweeps' bytes per solve follow the split
@@ -1392,7 +1392,7 @@ int bddc_autotune(bddc_handle_t h, int32_t nrhs, bddc_tuning_t* out, void* strea
     std::sort(best, best + 3);
     return best[1];
   };
-  bddc_tuning_t t{h->tune_stage_kb[0], h->tune_stage_kb[1], h->tune_coarse_rb_min, 64 << h->tune_tile_class[0],
+  bddc_tuning_t t{h->tune_stage_kb[0], h->tune_stage_kb[1], h->cs.rb_min, 64 << h->tune_tile_class[0],
                   64 << h->tune_tile_class[1], h->tune_overlap, h->tune_sym_stages[0], h->tune_sym_stages[1],
                   h->is.block_min_height, h->cs.use_level ? 1 : 0};
   cudaError_t ce = cudaSuccess;
@@ -1472,12 +1472,12 @@ int bddc_autotune(bddc_handle_t h, int32_t nrhs, bddc_tuning_t* out, void* strea
   }
   if (h->n_c && !h->coarse_dense && !h->coarse_cg && nrhs >= 2) {
     CUDA_TRY(cudaMemsetAsync(h->w.rc, 0, sizeof(double) * h->n_c * nrhs, st));
-    const int keep = h->tune_coarse_rb_min;
-    h->tune_coarse_rb_min = nrhs;   // blocked
+    const int keep = h->cs.rb_min;
+    h->cs.rb_min = nrhs;   // blocked
     const float blocked = timed([&] { return launch_coarse_solve(h, h->w, h->w.rc, h->w.uc, nrhs, st); });
-    h->tune_coarse_rb_min = 65;     // one row per unit
+    h->cs.rb_min = 65;     // one row per unit
     const float single = timed([&] { return launch_coarse_solve(h, h->w, h->w.rc, h->w.uc, nrhs, st); });
-    h->tune_coarse_rb_min = keep;
+    h->cs.rb_min = keep;
     if (blocked >= 0.0f && single >= 0.0f)
       t.coarse_rowblock_min_nrhs = blocked < single ? std::min(keep, (int)nrhs) : std::max(keep, (int)nrhs + 1);
   }
@@ -1485,7 +1485,7 @@ int bddc_autotune(bddc_handle_t h, int32_t nrhs, bddc_tuning_t* out, void* strea
   if (h->aux_stream[0] && h->n_c && !h->coarse_dense && h->nG_tot) {
     h->tune_stage_kb[0] = t.gemv_stage_kb_interior;
     h->tune_stage_kb[1] = t.gemv_stage_kb_interface;
-    h->tune_coarse_rb_min = t.coarse_rowblock_min_nrhs;
+    h->cs.rb_min = t.coarse_rowblock_min_nrhs;
     h->cs.use_level = t.coarse_level_launches == 1 && !h->cs.lv.empty();
     h->is.block_min_height = std::min(t.interior_block_height, h->is.levels);
     double* rz = nullptr;

@@ -234,12 +234,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_solve(CoarseArgs a) {
 // before a level runs, the pivots of its nodes collect theirs, r'_P = r_P - sum of
 // the contributions, in node order. That costs a second grid barrier per forward
 // level (about 2 us) and makes every product a plain one.
-// Measured against one row and column per warp (k_coarse_solve): 2863 coarse dofs,
-// 2 columns 118 us both, 8 columns 116 against 187, 64 columns 341 against 763;
-// interior forest of 160000 dofs, 4 columns: 0.55 against 2.54 ms. (4 rows x 8
-// columns per warp with float64 FMAs, the form before: 376 us for 32 columns on
-// 1011 coarse dofs, now 126.) What is left at 8 columns is latency: barriers and
-// one or two rounds of loads per level (the pipe is 23 % busy).
+// Measured against one row and column per warp (k_coarse_solve), whose time grows
+// with the columns where this one's is flat up to 8, in us at 2 / 4 / 8 / 64 columns:
+//   coarse dofs 2863    108 / 108 / 108 /  341   against 112 / 134 /  173 /  769
+//              10439    318 / 318 / 316 / 1199   against 247 / 327 /  550 / 3188
+//              25695    679 / 679 / 677 / 3630   against 464 / 745 / 1336 / 9058
+// and 2 / 4 / 8 columns of an interior forest:
+//   160000 dofs         551 / 549 / 553          against 1327 / 2541 / 4903
+//   640000 dofs        1557 / 1571 / 1599        against 4812 / 9618 / 18950
+// So it runs from 2 columns on, for coarse factors of more than kRbEntries entries
+// (between the first two) from 4 on. (4 rows x 8 columns per warp with float64 FMAs
+// took 376 us for 32 columns on 1011 coarse dofs, this form 126.) What is left at 8
+// columns is latency: barriers and one or two rounds of loads per level (the pipe is
+// 23 % busy on 2863 dofs).
+constexpr int64_t kRbEntries = 5000000;
 struct MmaArgs {
   const CNodeDev* nodes;
   const MUnit* units;
@@ -1319,6 +1327,7 @@ cudaError_t build_coarse_device(bddc_handle_s* h, const CoarseFactor& cf) {
   h->cs.bar = h->d_cbar;
   if ((e = build_sweeps(h, cf, h->cs, true, h->g_blocks, kSweepCoop, false)) != cudaSuccess) return e;
   h->c_nnz = h->cs.nnz;
+  h->cs.rb_min = h->c_nnz > kRbEntries ? 4 : 2;   // (the autotuner may move it)
   return cudaSuccess;
 }
 
@@ -1448,14 +1457,13 @@ cudaError_t launch_sweeps(bddc_handle_s* h, const SweepSet& S, const double* r, 
     h->launches++;
     return e;
   }
-  // the row-blocked form from tune_coarse_rb_min right-hand sides on (the
-  // autotuner may move the threshold)
+  // the row-blocked form from S.rb_min right-hand sides on
   cudaLaunchConfig_t cfg = {};
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   h->launches++;
-  if (nrhs >= h->tune_coarse_rb_min) {
+  if (nrhs >= S.rb_min) {
     MmaArgs m{S.nodes, S.munits, S.upd, S.order, S.mlvl, S.piv, S.cptr, S.cidx, S.F, S.B, r, rp, y, u, S.mcbuf, S.bar,
               h->d_err, S.levels, nrhs, extra, cycles};
     cfg.gridDim = dim3(narrow ? h->c_sms : S.mgrid);

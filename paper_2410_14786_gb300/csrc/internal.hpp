@@ -122,6 +122,7 @@ struct SweepSet {
   unsigned int* bar = nullptr;
   int64_t n = 0;                // dofs
   int levels = 0, grid = 0, mgrid = 0, g_blocks = 0;
+  int rb_min = 2;               // row-blocked form from this many right-hand sides on
   int g_fwd = 0, g_phases = 0;  // gather form: forward-type phases, all phases
   int64_t nnz = 0;              // stored entries of F and B
   int64_t g_entries = 0;        // stored entries of the gather form
@@ -427,7 +428,6 @@ struct bddc_handle_s {
   int tune_stage_kb[2] = {12, 12};   // streamed GEMV stage size: interior, interface operators
   int tune_sym_stages[2] = {4, 4};   // stages of the symmetric GEMV: interior, interface operators
   int tune_tile_class[2] = {1, 1};   // streamed GEMV row tile 64 << class: interior, interface
-  int tune_coarse_rb_min = 2;       // row-blocked coarse sweeps from this many right-hand sides on
   int tune_overlap = 0;              // interface operator concurrent with the coarse residual and solve
   // second stream of the apply and its fork / join events, one set per
   // capture sequence: [0] direct launches and the solve graph's prologue,
