@@ -40,11 +40,8 @@ cudaError_t dev_alloc(bddc_handle_s* h, T** p, size_t count) {
   *p = nullptr;
   if (count == 0) count = 1;
   void* v = nullptr;
-  cudaError_t e = cudaMalloc(&v, count * sizeof(T));
-  if (e == cudaSuccess) {
-    h->allocations.push_back(v);
-    *p = static_cast<T*>(v);
-  }
+  cudaError_t e = h->alloc(&v, count * sizeof(T));
+  if (e == cudaSuccess) *p = static_cast<T*>(v);
   return e;
 }
 
@@ -398,8 +395,7 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
     }
     const size_t bbytes = tc_operand_bytes(prec, std::max(h->tcB_cols_I, h->tcB_cols_G), h->nrhs_max);
     void* pB = nullptr;
-    CUDA_TRY(cudaMalloc(&pB, bbytes));
-    h->allocations.push_back(pB);
+    CUDA_TRY(h->alloc(&pB, bbytes));
     h->d_tcB = pB;
     h->use_tma = false;
   } else if (!h->full_operators && prec != BDDC_PREC_FP64 && h->nrhs_max == 1 && sgemv_tma_supported(prec, max_dim)) {
@@ -622,7 +618,7 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
     // the mixed forms sweep in float32 (an inexact interior solve inside
     // flexible PCG, as the low-precision dense operators are); FP64 in float64
     const bool c32 = h->precision != BDDC_PREC_FP64;
-    CUDA_TRY(build_sweeps(h, forest, h->is, h->nrhs_max > 1, 0, c32 ? kSweepLevel : kSweepBlock, c32));
+    CUDA_TRY(build_sweeps(h, forest, h->is, h->nrhs_max > 1, 0, c32 ? kSweepLevel : kSweepBlock, c32, false));
     // one interior solve at one column reads its coefficients once
     opbytes_I = sweep_read_1col(h->is);
     arena_bytes += (size_t)(h->is.g_entries * 12 + ((h->is.multi || h->is.block_form) ? h->is.nnz * 8 : 0));

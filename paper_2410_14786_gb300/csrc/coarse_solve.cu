@@ -997,9 +997,8 @@ __global__ void __launch_bounds__(kCgThreadsWide) k_coarse_cg(CgArgs a) {
 template <typename T>
 cudaError_t up(bddc_handle_s* h, T** dst, const std::vector<T>& v) {
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, std::max<size_t>(1, v.size()) * sizeof(T));
+  cudaError_t e = h->alloc(&p, std::max<size_t>(1, v.size()) * sizeof(T));
   if (e != cudaSuccess) return e;
-  h->allocations.push_back(p);
   *dst = static_cast<T*>(p);
   if (!v.empty()) e = cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
   return e;
@@ -1072,7 +1071,7 @@ cudaError_t build_coarse_cg_device(bddc_handle_s* h) {
 }
 
 cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, bool multi, int blocks_req,
-                         int form, bool coef32) {
+                         int form, bool coef32, bool one_row) {
   if (coef32 && form == kSweepCoop) return cudaErrorInvalidValue;
   const int L = cf.n_levels;
   S.levels = L;
@@ -1198,11 +1197,11 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
   // warp units: forward levels (L_PP^-1 rows, then one unit per receiving
   // position with its (node, M row) pairs in node order), then backward levels
   std::vector<CContrib> list;
-  std::vector<std::vector<int32_t>> contrib(cf.n);
+  std::vector<std::vector<int32_t>> contrib(one_row ? cf.n : 0);
   std::vector<int32_t> touched;
   std::vector<CUnit> units;
   std::vector<int32_t> lvl;
-  {
+  if (one_row) {
     lvl.assign(2 * (L + 1) + 1, 0);
     int32_t lcur = 0;
     for (int lv = 0; lv < L; ++lv) {
@@ -1291,7 +1290,7 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
   std::vector<double>().swap(B);
   if (!multi) return cudaSuccess;
   if ((e = up(h, &S.nodes, nodes)) != cudaSuccess) return e;
-  if ((e = up(h, &S.units, units)) != cudaSuccess) return e;
+  if (one_row && (e = up(h, &S.units, units)) != cudaSuccess) return e;
   if ((e = up(h, &S.munits, munits)) != cudaSuccess) return e;
   if ((e = up(h, &S.mlvl, mlvl)) != cudaSuccess) return e;
   if ((e = up(h, &S.piv, piv)) != cudaSuccess) return e;
@@ -1299,14 +1298,13 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
   if ((e = up(h, &S.cidx, cidx)) != cudaSuccess) return e;
   {
     void* cb = nullptr;
-    if ((e = cudaMalloc(&cb, std::max<size_t>(1, upd.size()) * h->nrhs_max * sizeof(double))) != cudaSuccess) return e;
-    h->allocations.push_back(cb);
+    if ((e = h->alloc(&cb, std::max<size_t>(1, upd.size()) * h->nrhs_max * sizeof(double))) != cudaSuccess) return e;
     S.mcbuf = static_cast<double*>(cb);
   }
-  if ((e = up(h, &S.list, list)) != cudaSuccess) return e;
+  if (one_row && (e = up(h, &S.list, list)) != cudaSuccess) return e;
   if ((e = up(h, &S.upd, upd)) != cudaSuccess) return e;
   if ((e = up(h, &S.order, cf.order)) != cudaSuccess) return e;
-  if ((e = up(h, &S.lvl, lvl)) != cudaSuccess) return e;
+  if (one_row && (e = up(h, &S.lvl, lvl)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_coarse_solve, kThreads, 0)) != cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorNotSupported;
@@ -1325,7 +1323,7 @@ cudaError_t build_coarse_device(bddc_handle_s* h, const CoarseFactor& cf) {
   cudaDeviceGetAttribute(&h->c_sms, cudaDevAttrMultiProcessorCount, dev);
   if (h->d_cbar == nullptr && (e = up(h, &h->d_cbar, std::vector<unsigned int>(2, 0u))) != cudaSuccess) return e;
   h->cs.bar = h->d_cbar;
-  if ((e = build_sweeps(h, cf, h->cs, true, h->g_blocks, kSweepCoop, false)) != cudaSuccess) return e;
+  if ((e = build_sweeps(h, cf, h->cs, true, h->g_blocks, kSweepCoop, false, true)) != cudaSuccess) return e;
   h->c_nnz = h->cs.nnz;
   h->cs.rb_min = h->c_nnz > kRbEntries ? 4 : 2;   // (the autotuner may move it)
   return cudaSuccess;
@@ -1463,7 +1461,7 @@ cudaError_t launch_sweeps(bddc_handle_s* h, const SweepSet& S, const double* r, 
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   h->launches++;
-  if (nrhs >= S.rb_min) {
+  if (nrhs >= S.rb_min) {   // (always without the one-row lists: rb_min is 2 then)
     MmaArgs m{S.nodes, S.munits, S.upd, S.order, S.mlvl, S.piv, S.cptr, S.cidx, S.F, S.B, r, rp, y, u, S.mcbuf, S.bar,
               h->d_err, S.levels, nrhs, extra, cycles};
     cfg.gridDim = dim3(narrow ? h->c_sms : S.mgrid);

@@ -560,5 +560,12 @@ struct bddc_handle_s {
   bool solve_graph_unsupported = false;
   cudaStream_t cap_stream = nullptr;       // private stream used only for capture
   int64_t launches = 0;                    // kernels launched so far
-  std::vector<void*> allocations;
+  std::vector<void*> allocations;          // freed with the handle; their bytes are in info.device_bytes
+  cudaError_t alloc(void** p, size_t bytes) {
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) return e;
+    allocations.push_back(*p);
+    info.device_bytes += (int64_t)bytes;
+    return e;
+  }
 };
