@@ -21,6 +21,9 @@ PRECISIONS = {"fp64": PREC_FP64, "fp32": PREC_FP32, "bf16": PREC_BF16, "tf32": P
 TENSOR_CORES = {"auto": _lib.TC_AUTO, True: _lib.TC_ON, False: _lib.TC_OFF}
 COARSE = {"auto": _lib.COARSE_AUTO, "dense": _lib.COARSE_DENSE, "sparse": _lib.COARSE_SPARSE, "cg": _lib.COARSE_CG}
 LOCAL = {"dense": _lib.LOCAL_DENSE, "sparse": _lib.LOCAL_SPARSE}
+# in the key of a tune cache: raised with every change of the kernels or thresholds that its entries choose
+# between, so that a choice measured on other kernels is measured again
+TUNED_KERNELS = 2
 
 
 @dataclass
@@ -61,7 +64,7 @@ class BDDC:
     autotune=True times the launch-parameter candidates on this handle's
     operators for nrhs_max columns and keeps the fastest (`autotune()`);
     tune_cache=path keeps those results in a JSON file keyed by the problem's
-    shape, partition and form, so a later handle for the same problem reuses
+    shape, partition and form and the kernels' revision, so a later handle for the same problem reuses
     them without measuring again; coarse_blocks: blocks of the one-column
     sparse coarse solve (0 = one per SM); full_operators=True stores the
     symmetric local operators in full where they would otherwise be stored
@@ -129,7 +132,7 @@ class BDDC:
         import hashlib
         import json
         import os
-        key = "|".join([f"dim{self.dim}", f"ne{self.ne}", f"nrhs{self.nrhs_max}", f"prec{self.precision}",
+        key = "|".join([f"kernels{TUNED_KERNELS}", f"dim{self.dim}", f"ne{self.ne}", f"nrhs{self.nrhs_max}", f"prec{self.precision}",
                         f"tc{self.info()['tensor_cores']}", f"sym{self.info()['symmetric_operators']}",
                         f"local{self.info()['local_solver']}",
                         hashlib.sha1(np.ascontiguousarray(part, dtype=np.int32).tobytes()).hexdigest()[:16]])
