@@ -16,10 +16,12 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <memory>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -165,9 +167,10 @@ inline void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std
   // a thread per 65536 entries, not more than asked for; no allocation in the threads
   const int nt = (int)std::max<int64_t>(1, std::min<int64_t>(threads, cur >> 16));
   std::vector<double> scratch((size_t)nt * (most + 1) * most);
+  std::atomic<size_t> next{0};
   auto work = [&](int t) {
-    double *S = &scratch[(size_t)t * (most + 1) * most], *size = S + (size_t)most * most;
-    for (size_t s = t; s < ops.size(); s += nt) {
+    double *S = scratch.data() + (size_t)t * (most + 1) * most, *size = S + (size_t)most * most;
+    for (size_t s; (s = next.fetch_add(1)) < ops.size();) {
       const int n = dims[s];
       if (n == 0) continue;
       int32_t* e = &P.rexp[voff[s]];
@@ -179,7 +182,13 @@ inline void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std
   };
   std::vector<std::thread> pool;
   pool.reserve(nt);
-  for (int t = 1; t < nt; ++t) pool.emplace_back(work, t);
+  for (int t = 1; t < nt; ++t) {
+    try {
+      pool.emplace_back(work, t);
+    } catch (const std::system_error&) {
+      break;   // the threads there are share the operators
+    }
+  }
   work(0);
   for (auto& t : pool) t.join();
 }

@@ -235,6 +235,39 @@ int main() {
       REQUIRE(worst <= std::max(worst64, 0x1p-53 + 1.25 * std::ldexp(1.0, kFxCertBits - 60)), "%s, %s: error %.2e against %.2e", o.name.c_str(), kinds[kind], worst, worst64);
     }
   }
+  // several operators in several threads: the same as each alone
+  {
+    std::vector<std::vector<double>> all;
+    std::vector<int> dims;
+    std::vector<int32_t> voff;
+    std::vector<uint8_t> drop;
+    int rows = 3;
+    for (int q = 0; q < 40; ++q) {
+      const Op& o = ops[q % ops.size()];
+      all.push_back(q == 17 ? std::vector<double>() : o.A);
+      dims.push_back(q == 17 ? 0 : o.n);
+      voff.push_back(rows);
+      rows += dims.back();
+    }
+    drop.assign(rows, 0);
+    for (int i = 5; i < rows; i += 50) drop[i] = 1;
+    FxPacked many;
+    fx_pack_lower(all, dims, voff, drop, 4, many);
+    for (size_t q = 0; q < all.size(); ++q) {
+      if (dims[q] == 0) continue;
+      FxPacked P;
+      fx_pack_lower({all[q]}, {dims[q]}, {0}, std::vector<uint8_t>(&drop[voff[q]], &drop[voff[q]] + dims[q]), 1, P);
+      const int64_t n = fx_packed_elems(dims[q]);
+      REQUIRE(many.off[q] % kFxTileElems == 0 &&
+                  std::memcmp(many.halves.get() + 2 * many.off[q], P.halves.get(), 8 * n) == 0 &&
+                  std::memcmp(many.values.get() + many.off[q], P.values.get(), 8 * n) == 0 &&
+                  std::memcmp(&many.rexp[voff[q]], P.rexp.data(), 4 * dims[q]) == 0 &&
+                  std::memcmp(&many.shift[many.off[q] / kFxTileElems], P.shift.data(), n / kFxTileElems) == 0,
+              "operator %zu packed with others", q);
+      for (int i = 0; i < dims[q]; ++i)
+        REQUIRE(!drop[voff[q] + i] || P.rexp[i] == kFxZero, "dropped row %d", i);
+    }
+  }
   // infinities and NaN: every row marked
   {
     FxPacked P;
