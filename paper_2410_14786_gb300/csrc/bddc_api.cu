@@ -441,23 +441,24 @@ int build_device(bddc_handle_s* h, HostSetup& hs, const bddc_problem_t* P) {
       double* values = nullptr;
       int8_t* shift = nullptr;
       cudaError_t e = dev_alloc(h, &halves, 2 * pk.elems);
-      if (e == cudaSuccess) e = cudaMemcpy(halves, pk.halves.get(), 8 * pk.elems, cudaMemcpyHostToDevice);
       if (e == cudaSuccess) e = dev_alloc(h, &values, pk.elems);
       if (e == cudaSuccess) e = cudaMemcpy(values, pk.values.get(), 8 * pk.elems, cudaMemcpyHostToDevice);
       if (e == cudaSuccess) e = upload(h, &rexp, pk.rexp);
       if (e == cudaSuccess) e = upload(h, &shift, pk.shift);
+      const std::vector<WorkItem> it = make_whole_items(pk.off, dims, voff, 8);
+      *n_items = (int)it.size();
+      if (e == cudaSuccess) e = upload(h, items, it);
+      h->fx[fam] = FxForm{halves, values, rexp, shift};
+      if (e == cudaSuccess) e = launch_fx_quantize(*items, *n_items, h->fx[fam], halves, nullptr);
       if (e != cudaSuccess) return e;
       arena_bytes += 16 * pk.elems;
-      h->fx[fam] = FxForm{halves, values, rexp, shift};
       h->use_fx[fam] = true;
-      const std::vector<WorkItem> it = make_whole_items(pk.off, dims, voff, 8);
       // (the float64 tiles are read for single rows only)
       *bytes = 0;
       for (int n : dims) *bytes += 8 * fx_packed_elems(n);
       *max_n = largest(dims);
       h->fx_share[fam] = 8.0 * fx_packed_elems(*max_n) / *bytes;
-      *n_items = (int)it.size();
-      return upload(h, items, it);
+      return cudaSuccess;
     };
     std::vector<int> dIf = dIop, dGf = dG;   // the operators kept in full
     if (prec == BDDC_PREC_FP64 && !h->full_operators) {

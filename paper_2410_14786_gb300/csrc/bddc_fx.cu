@@ -111,6 +111,29 @@ __device__ __forceinline__ int64_t shfl_xor64(int64_t v, int o) {
   return (int64_t)((uint32_t)lo) | ((int64_t)hi << 32);
 }
 
+// The fixed-point tiles of all operators from the float64 ones, an operator per
+// block at a time.
+__global__ void __launch_bounds__(256) k_fx_quantize(const WorkItem* __restrict__ items, int n_items,
+                                                     const double* __restrict__ values, const int32_t* __restrict__ rexp,
+                                                     const int8_t* __restrict__ shift, int2* __restrict__ halves) {
+  for (int u = blockIdx.x; u < n_items; u += gridDim.x) {
+    const WorkItem w = items[u];
+    const int n = w.ncols;
+    int64_t at = w.moff;
+    for (int I = 0; I * kFxTile < n; ++I)
+      for (int J = 0; J <= I; ++J, at += kFxTileElems) {
+        const int s = shift[at / kFxTileElems];
+        for (int e = threadIdx.x; e < kFxTileElems; e += blockDim.x) {
+          const int r = e / kFxTile, k = e % kFxTile, i = I * kFxTile + r, j = J * kFxTile + k;
+          int2 q;
+          fx_entry((uint64_t)__double_as_longlong(values[at + e]), i < n ? rexp[w.yoff + i] : 0,
+                   j < n ? rexp[w.yoff + j] : 0, s, q.x, q.y);
+          halves[at + fx_place(r, k)] = q;
+        }
+      }
+  }
+}
+
 // Shared memory of one block, in this order; T = tile rows of the largest
 // operator, npad its rows padded to whole tiles.
 struct FxSmem {
@@ -478,6 +501,13 @@ cudaError_t run_fx(const WorkItem* items, int n_items, int max_n, int S, const F
 
 bool fx_gemm_supported(int max_n) {
   return max_n <= kFxMaxBlocks * kFxTile && FxSmem(max_n, 1).total(kFxFewWarps, 1) <= (size_t)kFxSmemCap;
+}
+
+cudaError_t launch_fx_quantize(const WorkItem* items, int n_items, const FxForm& A, int32_t* halves, cudaStream_t st) {
+  if (n_items == 0) return cudaSuccess;
+  k_fx_quantize<<<std::min(n_items, 8 * num_sms()), 256, 0, st>>>(items, n_items, A.values, A.rexp, A.shift,
+                                                                  reinterpret_cast<int2*>(halves));
+  return cudaGetLastError();
 }
 
 cudaError_t launch_fx_gemm(const WorkItem* items, int n_items, int max_n, double share, const FxForm& A, const double* X,

@@ -1,5 +1,7 @@
-// Host packing of the float64 local operators for the fixed-point kernel
-// (bddc_fx.cu), free of CUDA so that it can be checked on the host.
+// Packing of the float64 local operators for the fixed-point kernel (bddc_fx.cu),
+// free of CUDA so that it can be checked on the host: the host forms the float64
+// tiles, their shifts and the row exponents, the device the fixed-point tiles from
+// them (fx_entry), which spares half of the packing and of the upload.
 //
 // An operator (symmetric: the packing takes (A + A^T) / 2) is stored as the
 // lower triangle of its tiles of 32 x 32: tile (I, J), J <= I, at position
@@ -43,8 +45,7 @@ inline int64_t fx_packed_elems(int n) { return (int64_t)fx_tiles(n) * kFxTileEle
 struct FxPacked {
   std::vector<int64_t> off;          // first entry of every operator (a multiple of kFxTileElems)
   int64_t elems = 0;
-  std::unique_ptr<int32_t[]> halves; // 2 elems: {low, high}
-  std::unique_ptr<double[]> values;  // elems
+  std::unique_ptr<double[]> values;  // the float64 tiles
   std::vector<int32_t> rexp;         // exponent of every row, at voff[s] + row (kFxZero: a row of zeros)
   std::vector<int8_t> shift;         // of every tile, padded to a multiple of 4
 };
@@ -122,27 +123,26 @@ inline int fx_tile_shift(const double* S, int n, int i0, int j0, const int32_t* 
   return s;
 }
 
-// The tiles of one operator.
-inline void fx_pack_operator(const double* S, int n, const int32_t* e, int32_t* halves, double* values, int8_t* shift) {
+// Fixed-point entry {low, high} of the value v in row i and column j (exponents
+// ei and ej) of a tile with shift s, and its place in the tile (in entries).
+FX_HD void fx_entry(uint64_t bits, int ei, int ej, int s, int32_t& lo, int32_t& hi) {
+  const int64_t q = bits << 1 ? fx_quantize(bits, kFxBits - ei - ej + s) : 0;
+  lo = fx_lo(q);
+  hi = fx_hi(q);
+}
+FX_HD int fx_place(int r, int k) { return r * kFxTile + ((k / 2) ^ (r & 7)) * 2 + k % 2; }
+
+// The float64 tiles of one operator and their shifts.
+inline void fx_pack_operator(const double* S, int n, const int32_t* e, double* values, int8_t* shift) {
   for (int I = 0; I * kFxTile < n; ++I)
     for (int J = 0; J <= I; ++J) {
-      const int i0 = I * kFxTile, j0 = J * kFxTile, s = fx_tile_shift(S, n, i0, j0, e);
-      *shift++ = (int8_t)s;
-      for (int r = 0; r < kFxTile; ++r, halves += 2 * kFxTile, values += kFxTile)
-        for (int k = 0; k < kFxTile; ++k) {
-          const bool in = i0 + r < n && j0 + k < n;
-          const double v = in ? S[(size_t)(i0 + r) * n + j0 + k] : 0.0;
-          int64_t q = 0;
-          if (v != 0.0) {
-            uint64_t b;
-            std::memcpy(&b, &v, 8);
-            q = fx_quantize(b, kFxBits - e[i0 + r] - e[j0 + k] + s);
-          }
-          const int at = ((k / 2) ^ (r & 7)) * 2 + k % 2;
-          halves[2 * at] = fx_lo(q);
-          halves[2 * at + 1] = fx_hi(q);
-          values[k] = v;
-        }
+      const int i0 = I * kFxTile, j0 = J * kFxTile, nj = std::min(kFxTile, n - j0);
+      *shift++ = (int8_t)fx_tile_shift(S, n, i0, j0, e);
+      for (int r = 0; r < kFxTile; ++r, values += kFxTile) {
+        const int m = i0 + r < n ? nj : 0;
+        if (m) std::memcpy(values, S + (size_t)(i0 + r) * n + j0, sizeof(double) * m);
+        std::fill(values + m, values + kFxTile, 0.0);
+      }
     }
 }
 
@@ -160,8 +160,7 @@ inline void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std
     most = std::max(most, dims[s]);
   }
   P.elems = std::max<int64_t>(cur, kFxTileElems);
-  P.halves.reset(new int32_t[2 * P.elems]);   // (every entry is written below, by the threads)
-  P.values.reset(new double[P.elems]);
+  P.values.reset(new double[P.elems]);   // (every entry is written below, by the threads)
   P.rexp.assign((size_t)std::max<int64_t>(rows, 1), 0);
   P.shift.assign((size_t)(P.elems / kFxTileElems + 3) / 4 * 4, 0);
   // a thread per 65536 entries, not more than asked for; no allocation in the threads
@@ -176,8 +175,7 @@ inline void fx_pack_lower(const std::vector<std::vector<double>>& ops, const std
       int32_t* e = &P.rexp[voff[s]];
       fx_symmetric_part(ops[s].data(), n, drop.empty() ? nullptr : &drop[voff[s]], S);
       fx_row_exponents(S, n, e, size);
-      fx_pack_operator(S, n, e, P.halves.get() + 2 * P.off[s], P.values.get() + P.off[s],
-                       &P.shift[P.off[s] / kFxTileElems]);
+      fx_pack_operator(S, n, e, P.values.get() + P.off[s], &P.shift[P.off[s] / kFxTileElems]);
     }
   };
   std::vector<std::thread> pool;

@@ -36,6 +36,8 @@ cudaError_t launch_sgemv_tma(int precision, const WorkItem* items, int n_items, 
 // as for the symmetric GEMV above; share: the largest operator's part of all
 // operators' entries).
 bool fx_gemm_supported(int max_n);
+// Setup: the fixed-point tiles (halves) from the float64 ones, exponents and shifts of A.
+cudaError_t launch_fx_quantize(const WorkItem* items, int n_items, const FxForm& A, int32_t* halves, cudaStream_t st);
 cudaError_t launch_fx_gemm(const WorkItem* items, int n_items, int max_n, double share, const FxForm& A, const double* X,
                            double* Y, const int32_t* yscatter, int nrhs, int32_t* err, cudaStream_t st);
 // stage_kb: target bytes of one shared-memory stage, in KB (1..64; 12 by default,

@@ -52,10 +52,27 @@ static std::vector<double> inverse(int dim, int m, const std::function<double(in
   return A;
 }
 
+// The fixed-point tiles of one operator {low, high}, as the device forms them.
+static std::vector<int32_t> halves(const FxPacked& P, int n) {
+  std::vector<int32_t> out(2 * fx_packed_elems(n));
+  for (int I = 0; I * kFxTile < n; ++I)
+    for (int J = 0; J <= I; ++J)
+      for (int r = 0; r < kFxTile; ++r)
+        for (int k = 0; k < kFxTile; ++k) {
+          const int t = fx_tile_at(I, J), i = I * kFxTile + r, j = J * kFxTile + k;
+          uint64_t b;
+          std::memcpy(&b, &P.values[(size_t)t * kFxTileElems + r * kFxTile + k], 8);
+          int32_t* at = &out[2 * ((size_t)t * kFxTileElems + fx_place(r, k))];
+          fx_entry(b, i < n ? P.rexp[i] : 0, j < n ? P.rexp[j] : 0, P.shift[t], at[0], at[1]);
+        }
+  return out;
+}
+
 // One product in fixed point, as the kernel forms it; used[i]: row i holds.
 static void product(const FxPacked& P, int n, const std::vector<double>& x, std::vector<double>& y,
                     std::vector<char>& used) {
   const int T = (n + kFxTile - 1) / kFxTile;
+  const std::vector<int32_t> tiles = halves(P, n);
   std::vector<int> E(T, kFxZero);
   std::vector<int32_t> xh(T * kFxTile, 0), xl(T * kFxTile, 0);
   auto bits = [](double v) { uint64_t b; std::memcpy(&b, &v, 8); return b; };
@@ -88,12 +105,12 @@ static void product(const FxPacked& P, int n, const std::vector<double>& x, std:
       uint32_t tf = 0, t0 = 0, size = 0;
       int32_t t1 = 0;
       for (int J = 0; J < T; ++J) {
-        const int32_t* tile = P.halves.get() + 2 * (P.off[0] + (int64_t)fx_tile_at(I, J) * kFxTileElems);
+        const int32_t* tile = &tiles[2 * (int64_t)fx_tile_at(I, J) * kFxTileElems];
         int64_t h[2] = {0, 0}, m[2] = {0, 0};
         for (int k = 0; k < kFxTile; ++k) {
           // row r of tile (I, J), or column r of tile (J, I): halves even / odd, or lower / upper
           const int row = J <= I ? r : k, col = J <= I ? k : r, half = J <= I ? k & 1 : k >> 4;
-          const int at = row * kFxTile + ((col / 2) ^ (row & 7)) * 2 + col % 2;
+          const int at = fx_place(row, col);
           const int64_t al = tile[2 * at], ah = tile[2 * at + 1];
           h[half] += ah * xh[J * kFxTile + k];
           m[half] += ah * xl[J * kFxTile + k] + al * xh[J * kFxTile + k];
@@ -172,6 +189,7 @@ int main() {
     const int n = o.n;
     FxPacked P;
     fx_pack_lower({o.A}, {n}, {0}, {}, 1, P);
+    const std::vector<int32_t> tiles = halves(P, n);
     // the packed entries: float64 exactly, fixed point to 2^-59 of the tile's scale
     for (int i = 0; i < n; ++i)
       for (int j = 0; j < n; ++j) {
@@ -180,8 +198,8 @@ int main() {
         const int row = i % kFxTile, col = j % kFxTile, t = fx_tile_at(I, J);
         const double s = 0.5 * (o.A[i * n + j] + o.A[j * n + i]);
         REQUIRE(P.values[(size_t)t * kFxTileElems + row * kFxTile + col] == s, "%s: value", o.name.c_str());
-        const int64_t at = (int64_t)t * kFxTileElems + row * kFxTile + ((col / 2) ^ (row & 7)) * 2 + col % 2;
-        const int64_t q = (int64_t)P.halves[2 * at + 1] * (1ll << kFxLow) + P.halves[2 * at];
+        const int64_t at = (int64_t)t * kFxTileElems + fx_place(row, col);
+        const int64_t q = (int64_t)tiles[2 * at + 1] * (1ll << kFxLow) + tiles[2 * at];
         if (s == 0.0) {
           REQUIRE(q == 0, "%s: zero", o.name.c_str());
           continue;
@@ -259,7 +277,6 @@ int main() {
       fx_pack_lower({all[q]}, {dims[q]}, {0}, std::vector<uint8_t>(&drop[voff[q]], &drop[voff[q]] + dims[q]), 1, P);
       const int64_t n = fx_packed_elems(dims[q]);
       REQUIRE(many.off[q] % kFxTileElems == 0 &&
-                  std::memcmp(many.halves.get() + 2 * many.off[q], P.halves.get(), 8 * n) == 0 &&
                   std::memcmp(many.values.get() + many.off[q], P.values.get(), 8 * n) == 0 &&
                   std::memcmp(&many.rexp[voff[q]], P.rexp.data(), 4 * dims[q]) == 0 &&
                   std::memcmp(&many.shift[many.off[q] / kFxTileElems], P.shift.data(), n / kFxTileElems) == 0,
