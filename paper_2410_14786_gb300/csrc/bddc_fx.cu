@@ -23,12 +23,13 @@
 // result depends on no order.
 //
 // Rows whose certificate does not hold (fx.hpp) are listed at the unit's end and
-// summed in float64, a warp each, from the float64 form of the tiles: none or a
-// few in 10^4 for dense operands, 0.3 to 2 % in the iterations of a solve with
-// lognormal conductivities (up to a quarter of one operator), most of them for an
+// summed in float64, a warp each, from the float64 form of the tiles: a few in 10^5
+// for dense operands, 0.1 to 0.6 % in the iterations of a solve with lognormal
+// conductivities (up to a tenth of one operator: that solve takes 27.7 ms on 96^3
+// elements, 25.9 without a certificate and 49.2 in float64), a third or so for an
 // operand with one entry.
 //
-// Measured on 1728 operators of 343 rows at one column: 174 us, 5.4 TB/s of stored
+// Measured on 1728 operators of 343 rows at one column: 172 us, 5.4 TB/s of stored
 // entries (the float64 kernel: 401 us); on 512 of them at 8 columns 322 us, half
 // of the integer multiply-add rate (the float64 kernel: 1085 us). (8 warps of 3
 // tiles in flight took 10 % longer than 12 of 2, 6 of 4 30 %; row-major triangles
@@ -280,10 +281,26 @@ __global__ void __launch_bounds__(kFxWarps * 32, 1)
     for (int b = warp; b < NC * ldT; b += nw) {
       const int k = NC == 1 ? 0 : b / ldT, i = (b - k * ldT) * kFxTile + lane, at = k * npad + i;
       const uint64_t v = (uint64_t)__double_as_longlong(xraw[at]);
-      const int ei = xexp[i], E = __reduce_max_sync(0xffffffffu, fx_scaled_exponent(v, ei));
-      int64_t q = 0;
-      if (E != kFxZero && E != kFxNonFinite && ei != kFxZero) q = fx_quantize(v, kFxBits - E + ei);
-      xq[at] = make_int2(fx_lo(q), fx_hi(q));
+      const int ei = xexp[i];
+      int E = __reduce_max_sync(0xffffffffu, fx_scaled_exponent(v, ei));
+      int2 h = make_int2(0, 0);
+      if (E != kFxZero && E != kFxNonFinite) {
+        auto round = [&]() {
+          const int64_t q = ei != kFxZero ? fx_quantize(v, kFxBits - E + ei) : 0;
+          h = make_int2(fx_lo(q), fx_hi(q));
+        };
+        round();
+        const uint32_t part = fx_part(h.y), all = __reduce_add_sync(0xffffffffu, part);
+        if (fx_half_exceeds(all)) {   // the lower and upper, the even and odd half
+          const uint32_t low = __reduce_add_sync(0xffffffffu, lane < 16 ? part : 0);
+          const uint32_t even = __reduce_add_sync(0xffffffffu, lane & 1 ? 0 : part);
+          if (fx_half_exceeds(max(max(low, all - low), max(even, all - even)))) {
+            ++E;
+            round();
+          }
+        }
+      }
+      xq[at] = h;
       if (lane == 0) xe[b] = E;
     }
   };
@@ -468,7 +485,8 @@ __global__ void __launch_bounds__(kFxWarps * 32, 1)
     }
     if (has_next) row_scales(u + gridDim.x, par ^ 1);
     __syncthreads();                          // C: sums clear; the next top, far_list and far_count complete
-    for (int q = warp; q < min(far_count[par], kFarList); q += nw) row64(far_list[q]);
+    // (from the last warp on: the tiles are dealt from the first one on)
+    for (int q = nw - 1 - warp; q < min(far_count[par], kFarList); q += nw) row64(far_list[q]);
     par ^= 1;
     if (tid == 0) far_count[par] = 0;         // (added to after the next B)
     if (u + 2 * (int)gridDim.x < n_units) prefetch_operand(u + 2 * gridDim.x, par ^ 1);

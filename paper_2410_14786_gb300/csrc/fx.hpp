@@ -15,11 +15,12 @@
 // Blocks. An operand's blocks are kFxBlock consecutive values, an operator's
 // tiles of kFxBlock x kFxBlock entries, each with its own exponent; a block sum
 // is formed of one block of the operand and a row (or column) of one tile. A
-// value is exact unless it is below 2^-6 of its block's scale (59 bits hold 53
-// there), else its error is 2^-60 of that scale. A tile's scale is such that the
-// absolute sum of a row or column is at most kFxBlockSum in its units, which
-// keeps the sum of h h' within 2^62 and that of h l' within 2^60; l h' adds at most
-// 2^58 per product, 16 of them to a 64-bit sum.
+// value is exact unless it is below 2^-7 of its block's scale (60 bits hold 53
+// there), else its error is 2^-61 of that scale. A tile's scale is such that the
+// absolute sum of a row or column is at most kFxBlockSum in its units, an operand
+// block's such that no half of it (16 values, of one 64-bit sum) has an absolute
+// sum above kFxHalfSum: that keeps a sum of h h' within 2^62, of h l' within 2^61
+// and of l h' within 2^62.
 //
 // Rows. A block sum joins the row's total in the unit of the row's largest
 // block (fx_shift_sum), as an integer of 2^kFxShift times the unit of h h' and a
@@ -47,17 +48,18 @@
 
 namespace bddc {
 
-constexpr int kFxBits = 59;       // magnitude bits of a value
-constexpr int kFxLow = 29;        // bits of the low half
+constexpr int kFxBits = 60;       // magnitude bits of a value
+constexpr int kFxLow = 30;        // bits of the low half
 constexpr int kFxBlock = 32;      // products of one block (16 per 64-bit sum, two sums)
 constexpr int kFxBlockSum = 4;    // largest absolute sum of a row or column of a tile, in units of its scale
+constexpr int kFxHalfSum = 8;     // largest absolute sum of half an operand block, in units of its scale
 constexpr int kFxMaxBlocks = 124; // blocks of a row
 constexpr int kFxShift = 13;      // low bits of a block's h h' sum that go to the fraction
 constexpr int kFxFrac = 24;       // bits of the fraction
 constexpr int kFxLimb = 25;       // bits of the low limb of a total
 constexpr int kFxZero = -8192;    // exponent of a zero
 constexpr int kFxNonFinite = 8192;   // exponent of an infinity or NaN
-constexpr int kFxCertBits = 6;    // a row's magnitude is at least 2^-this of its scale
+constexpr int kFxCertBits = 7;    // a row's magnitude is at least 2^-this of its scale
 constexpr int kFxCertUnit = 20;   // magnitudes are in units of 2^-this of full scale
 constexpr int kFxScaleBits = 12;  // blocks further below a row's largest don't count in its mean scale
 constexpr int kFxZeroTile = 127;  // shift of a tile of zeros
@@ -85,7 +87,7 @@ FX_HD int64_t fx_quantize(uint64_t bits, int add) {
 }
 
 // The same for the words {lo, hi} of a finite x with |x| < 2^E, rounded to
-// `bits` bits and in fewer instructions: round(x 2^(bits - E)), 54 <= bits <= 59.
+// `bits` bits and in fewer instructions: round(x 2^(bits - E)), 54 <= bits <= 60.
 // E is at least -1021, so that 0 and subnormal numbers fit too.
 FX_HD int64_t fx_quantize_words(int32_t lo, int32_t hi, int E, int bits = kFxBits) {
   const int e = (hi >> 20) & 0x7ff;
@@ -140,6 +142,9 @@ FX_HD int fx_scaled_exponent(uint64_t bits, int e) {
   const int x = fx_exponent(bits);
   return x == kFxNonFinite || x == kFxZero ? x : e == kFxZero ? kFxZero : x + e;
 }
+// Whether half an operand block with this sum of fx_part(h) exceeds kFxHalfSum.
+FX_HD uint32_t fx_part(int32_t h) { return (uint32_t)(h < 0 ? -h : h) >> 4; }
+FX_HD bool fx_half_exceeds(uint32_t sum) { return sum > (uint32_t)kFxHalfSum << (kFxBits - kFxLow - 4); }
 // Scale of the products of an operand block (exponent E) and a tile (shift s).
 FX_HD int fx_block_scale(int E, int s) {
   return E == kFxNonFinite ? E : E == kFxZero || s == kFxZeroTile ? kFxZero : E - s;
