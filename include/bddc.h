@@ -267,9 +267,11 @@ int bddc_apply(bddc_handle_t h, const double *r, double *z, int32_t nrhs, void *
  * other teardown of the device's primary context. Every call on every handle of
  * a device shares the one array, and no part of it needs to start at zero
  * (each call writes every element it reads before reading it): calls that
- * overlap on the GPU, on any streams, race and give wrong results. The call
- * does not modify the handle; as for every call on a handle, no other host
- * thread may use the same handle meanwhile. */
+ * overlap on the GPU, on any streams, race and give wrong results. The
+ * call's other buffers are the handle's (the packed operands of the tensor-
+ * core and blocked float32 products, the contribution buffer and barrier of
+ * the coarse sweeps); as for every call on a handle, no other host thread may
+ * use the same handle meanwhile. */
 int bddc_apply_static_scratch(bddc_handle_t h, const double *r, double *z, int32_t nrhs,
                               void *stream);
 

@@ -68,7 +68,8 @@ class BDDC:
     them without measuring again; coarse_blocks: blocks of the one-column
     sparse coarse solve (0 = one per SM); full_operators=True stores the
     symmetric local operators in full where they would otherwise be stored
-    as lower triangles (fp32 / bf16 on the CUDA cores with nrhs_max = 1);
+    as lower triangles (fp64, in fixed point with float64 beside it; fp32 /
+    bf16 on the CUDA cores with nrhs_max = 1);
     history: PCG iterations whose scalars (||r_k||, alpha_k, beta_k) the
     handle keeps for `pcg_history()` (0 = none); coarse="cg" solves the
     coarse system inexactly by plain CG (the paper's choice) to
