@@ -159,7 +159,7 @@ typedef struct {
                               the FP32 and BF16 forms on the CUDA cores with nrhs_max = 1
                               (about half the bytes, applied by the symmetric streamed
                               GEMV), and in the FP64 form up to 3968 rows (many operators
-                              of fewer than about 100 rows excepted), in block fixed
+                              of fewer than about 60 rows excepted), in block fixed
                               point with the float64 triangles beside it (together about
                               the bytes of the full operators). A row of a product is
                               used in fixed point where it is as accurate as the float64

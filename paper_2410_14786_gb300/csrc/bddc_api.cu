@@ -208,13 +208,13 @@ std::vector<WorkItem> make_whole_items(const std::vector<int64_t>& off, const st
 }
 
 // Whether a family of float64 operators runs in block fixed point. A unit of that
-// kernel is a whole operator, at the cost of three block barriers and a chain of
-// loads (about 3 us), which many small operators don't earn back against the
-// streamed GEMV's row tiles: at one column 4096 operators of 27 rows take 124 us
-// against 21, 1728 of 64 rows 59 against 23, of 125 rows 67 against 67, of 136 rows
-// 68 against 106; more columns favour fixed point earlier (4096 operators of 89
-// rows: 129 against 83 us at one column, 166 against 160 at 2, 254 against 397 at
-// 4; 576 of 49 rows 56 against 48 at 8, of 81 rows 60 against 105). Up to about 32
+// kernel is a whole operator in whole tiles, at the cost of three block barriers and
+// a chain of loads, which many small operators don't earn back against the streamed
+// GEMV's row tiles: at one column 4096 operators of 27 rows take 40 us against 21,
+// 576 of 49 rows 15 against 11, of 81 rows 17 both, 1728 of 64 rows 24 both, 4096 of
+// 89 rows 68 against 84; more columns favour fixed point earlier (1728 of 64 rows 30
+// against 40 us at 2 columns; 576 of 38 rows 21 both, of 49 rows 22 against 28 at 4;
+// 1600 of 25 rows 42 against 56, 144 of 44 rows 18 against 14 at 8). Up to about 32
 // operators either form is one wave of launch latency.
 bool use_fx_family(const std::vector<int>& dims, int nrhs_max) {
   int n = 0, count = 0;
@@ -224,7 +224,7 @@ bool use_fx_family(const std::vector<int>& dims, int nrhs_max) {
     count += d > 0;
     sq += (double)d * d;
   }
-  const double least = nrhs_max == 1 ? 125.0 : nrhs_max < 4 ? 100.0 : nrhs_max < 8 ? 80.0 : 70.0;
+  const double least = nrhs_max == 1 ? 64.0 : nrhs_max < 4 ? 56.0 : nrhs_max < 8 ? 40.0 : 32.0;
   return n > 0 && fx_gemm_supported(n) && (count <= 32 || sq >= least * least * count);
 }
 

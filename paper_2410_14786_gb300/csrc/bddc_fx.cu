@@ -11,30 +11,27 @@
 // on the integer multiply-adds are the larger part (3 per full entry and column
 // against one float64 FMA at a sixteenth of their rate).
 //
-// Split. One block of 12 warps owns one unit, an operator and up to NC columns,
-// at a time; the tiles are dealt
-// to the warps, and every warp streams its own ones through a private ring of
-// bulk copies that runs on into the next unit, so no warp waits for another
-// one but at a unit's end. A tile is read twice from shared
-// memory, so that neither use needs a reduction across the warp: once with a
-// row per lane (its row's products with x_J), once with two columns per lane
-// (the products with x_I of the mirrored tile). The sums go to shared
-// memory with 32-bit integer atomics that nothing waits for: exact, so the
-// result depends on no order.
+// Split. One block of up to 12 warps owns one unit, an operator and up to NC
+// columns, at a time; the tiles are dealt to the warps, and every warp streams its
+// own ones through a private ring of bulk copies that runs on into the next unit,
+// so no warp waits for another one but at a unit's end. A tile is read twice from
+// shared memory, so that neither use needs a reduction across the warp: once with a
+// row per lane (its row's products with x_J), once with two columns per lane (the
+// products with x_I of the mirrored tile). The sums go to shared memory with 32-bit
+// integer atomics that nothing waits for: exact, so the result depends on no order.
 //
 // Rows whose certificate does not hold (fx.hpp) are listed at the unit's end and
 // summed in float64, a warp each, from the float64 form of the tiles: a few in 10^5
 // for dense operands, 0.1 to 0.6 % in the iterations of a solve with lognormal
-// conductivities (up to a tenth of one operator: that solve takes 27.7 ms on 96^3
-// elements, 25.9 without a certificate and 49.2 in float64), a third or so for an
+// conductivities (up to a tenth of one operator: that solve takes 26.9 ms on 96^3
+// elements, 25.9 without a certificate and 49.1 in float64), a third or so for an
 // operand with one entry.
 //
-// Measured on 1728 operators of 343 rows at one column: 172 us, 5.4 TB/s of stored
+// Measured on 1728 operators of 343 rows at one column: 165 us, 5.6 TB/s of stored
 // entries (the float64 kernel: 401 us); on 512 of them at 8 columns 322 us, half
-// of the integer multiply-add rate (the float64 kernel: 1085 us). (8 warps of 3
-// tiles in flight took 10 % longer than 12 of 2, 6 of 4 30 %; row-major triangles
-// with whole rows per warp 270 to 430 us: rows of many lengths cost more
-// instructions in control and reductions than in products.)
+// of the integer multiply-add rate (the float64 kernel: 1085 us). (Row-major
+// triangles with whole rows per warp took 270 to 430 us: rows of many lengths cost
+// more instructions in control and reductions than in products.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,11 +45,12 @@
 namespace bddc {
 
 namespace {
-constexpr int kFxWarps = 12;                // of a block; kFxFewWarps where more rings don't fit
+constexpr int kFxWarps = 12;                // of a block at most; kFxFewWarps where more rings don't fit
 constexpr int kFxFewWarps = 8;
 constexpr int kFxTileBytes = kFxTileElems * 8;
 constexpr int kFxMaxSlots = 2;              // tiles in flight per warp
 constexpr int kFxSmemCap = 225 * 1024;      // of 227 KB, beside the static ones
+constexpr int kFxSmemSm = 228 * 1024;       // of an SM; 1 KB of it is taken by every block
 constexpr int kFarList = 256;
 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
@@ -503,14 +501,30 @@ template <int NC>
 cudaError_t run_fx(const WorkItem* items, int n_items, int max_n, int S, const FxForm& A, const double* X, double* Y,
                    const int32_t* yscatter, int nrhs, int32_t* err, cudaStream_t st) {
   const FxSmem L(max_n, NC);
+  const FxUnits U{n_items, (nrhs + NC - 1) / NC, S};
+  const int64_t units = (int64_t)n_items * U.ncb * S;
   auto fits = [&](int nw, int nst) { return L.total(nw, nst) <= (size_t)kFxSmemCap; };
-  const int nst = fits(kFxWarps, kFxMaxSlots) ? kFxMaxSlots : 1, nw = fits(kFxWarps, nst) ? kFxWarps : kFxFewWarps;
+  auto blocks = [&](int nw) { return std::min(kFxWarps / nw, (int)(kFxSmemSm / (L.total(nw, kFxMaxSlots) + 1024))); };
+  // Warps of a block: as many as the largest operator has tiles, up to 12, in one
+  // block per SM; narrower blocks, several to an SM, where there are more units than
+  // SMs: the waits at a unit's end and its chain of loads then overlap with other
+  // units. Three (two) blocks of 4 warps for operators of up to 6 tile rows, two of
+  // 6 warps for larger ones at one or two columns, as far as both fit (1728
+  // operators, one column: 64 rows 24 us against 59 with 12 warps, 125 rows 40
+  // against 67, 343 rows 165 against 171; 4 columns of 125 rows 110 against 128;
+  // 8 columns of 196 rows, where one block of 4 warps fits, 613 against 397).
+  int nw = std::max(4, std::min(kFxWarps, fx_tiles(max_n)));
+  if (units > num_sms()) {
+    if (L.T <= 6 && blocks(4) >= 2) nw = 4;
+    else if (NC <= 2 && nw > 6 && blocks(6) >= 2) nw = 6;
+  }
+  const int nst = fits(nw, kFxMaxSlots) ? kFxMaxSlots : 1;
+  if (!fits(nw, nst)) nw = kFxFewWarps;
   const size_t smem = L.total(nw, nst);
   cudaError_t e = cudaFuncSetAttribute(k_fx_gemm<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const FxUnits U{n_items, (nrhs + NC - 1) / NC, S};
-  // one block per SM: the rings take its shared memory
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)n_items * U.ncb * S, num_sms()));
+  const int per_sm = nst == kFxMaxSlots ? std::max(1, blocks(nw)) : 1;
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(units, (int64_t)per_sm * num_sms()));
   k_fx_gemm<NC><<<grid, nw * 32, smem, st>>>(items, U, A, X, Y, yscatter, nrhs, nst, max_n, err);
   return cudaGetLastError();
 }

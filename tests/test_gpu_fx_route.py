@@ -17,7 +17,7 @@ def _built():
 
 # (dim, elements, subdomains per direction, columns): interiors and interfaces of
 # about 25 and 23, 27 and 76, 225 and 55, 343 and 290 rows
-@pytest.mark.parametrize("dim,ne,nsub,nrhs,families", [(2, 72, 12, 1, 0), (2, 72, 12, 8, 0), (3, 24, 6, 1, 0),
+@pytest.mark.parametrize("dim,ne,nsub,nrhs,families", [(2, 72, 12, 1, 0), (2, 72, 12, 8, 0), (3, 24, 6, 1, 1),
                                                        (3, 24, 6, 8, 1), (2, 96, 6, 1, 1), (3, 32, 4, 1, 2)])
 def test_families(dim, ne, nsub, nrhs, families):
     from paper_2410_14786_gb300 import BDDC
