@@ -384,7 +384,7 @@ cudaError_t run_tma(const WorkItem* items, int n_items, int max_lda, const T* ar
   const int stage_bytes = stage_size<T, NRB>(max_lda, stage_kb);
   const size_t smem = block_smem<T, NRB>(stage_bytes, max_lda);
   auto kern = k_bgemv_tma<T, NRB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTmaThreads, smem);
@@ -788,7 +788,7 @@ cudaError_t run_sym(const WorkItem* items, int n_items, int max_n, const T* aren
   const size_t smem = sym_smem<T, K>(stage_bytes, nst, max_n);
   if (smem > (size_t)kSymSmemCap) return cudaErrorInvalidValue;
   auto kern = k_sgemv_tma<T, K>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTmaThreads, smem);

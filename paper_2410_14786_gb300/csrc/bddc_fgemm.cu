@@ -194,7 +194,7 @@ cudaError_t run_fgemm(const FgOperators& F, const float* P, int64_t cstride, dou
   static_assert(Sh::RT == 32 << cls, "row tiles of the item lists");
   constexpr int smem = kFgStages * Sh::stage;
   auto kern = k_fgemm<NW, CB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const int ncg = (nrhs + kFgCols * CB - 1) / (kFgCols * CB);
   int per_sm = 0;

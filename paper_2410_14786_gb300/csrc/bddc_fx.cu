@@ -49,7 +49,7 @@ constexpr int kFxWarps = 12;                // of a block at most; kFxFewWarps w
 constexpr int kFxFewWarps = 8;
 constexpr int kFxTileBytes = kFxTileElems * 8;
 constexpr int kFxMaxSlots = 2;              // tiles in flight per warp
-constexpr int kFxSmemCap = 225 * 1024;      // of 227 KB, beside the static ones
+constexpr size_t kFxSmemCap = kSmemMost;
 constexpr int kFxSmemSm = 228 * 1024;       // of an SM; 1 KB of it is taken by every block
 constexpr int kFarList = 256;
 
@@ -182,10 +182,10 @@ __global__ void __launch_bounds__(kFxWarps * 32, 1)
   const FxSmem L(max_n, NC);
   const int npad = L.npad, ldT = L.T, n_units = U.count();
   const int2* arena = reinterpret_cast<const int2*>(A.halves);
-  int2* xq = reinterpret_cast<int2*>(smem + (size_t)(blockDim.x >> 5) * nst * kFxTileBytes);   // operand halves [NC][npad]
-  double* xraw = reinterpret_cast<double*>(xq + NC * npad);                           // next operand
+  int2* xq = reinterpret_cast<int2*>(smem + (size_t)(blockDim.x >> 5) * nst * kFxTileBytes);   // operand [NC][npad]
+  double* xraw = reinterpret_cast<double*>(xq + NC * npad);                                    // next operand
   uint64_t* bars = reinterpret_cast<uint64_t*>(xraw + NC * npad);
-  uint32_t* sums = reinterpret_cast<uint32_t*>(bars + (blockDim.x >> 5) * nst);   // totals and magnitudes [4][NC][npad]
+  uint32_t* sums = reinterpret_cast<uint32_t*>(bars + (blockDim.x >> 5) * nst);   // totals, magnitudes [4][NC][npad]
   int32_t* xexp = reinterpret_cast<int32_t*>(sums + 4 * NC * npad);      // row exponents of the next operand
   int32_t* xe = xexp + npad;                                             // exponents of the operand's blocks [NC][T]
   int32_t* top_of = xe + NC * ldT;                                       // of this unit and the next: unit of a tile
@@ -503,7 +503,7 @@ cudaError_t run_fx(const WorkItem* items, int n_items, int max_n, int S, const F
   const FxSmem L(max_n, NC);
   const FxUnits U{n_items, (nrhs + NC - 1) / NC, S};
   const int64_t units = (int64_t)n_items * U.ncb * S;
-  auto fits = [&](int nw, int nst) { return L.total(nw, nst) <= (size_t)kFxSmemCap; };
+  auto fits = [&](int nw, int nst) { return L.total(nw, nst) <= kFxSmemCap; };
   auto blocks = [&](int nw) { return std::min(kFxWarps / nw, (int)(kFxSmemSm / (L.total(nw, kFxMaxSlots) + 1024))); };
   // Warps of a block: as many as the largest operator has tiles, up to 12, in one
   // block per SM; narrower blocks, several to an SM, where there are more units than
@@ -521,7 +521,7 @@ cudaError_t run_fx(const WorkItem* items, int n_items, int max_n, int S, const F
   const int nst = fits(nw, kFxMaxSlots) ? kFxMaxSlots : 1;
   if (!fits(nw, nst)) nw = kFxFewWarps;
   const size_t smem = L.total(nw, nst);
-  cudaError_t e = cudaFuncSetAttribute(k_fx_gemm<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_fx_gemm<NC>, smem);
   if (e != cudaSuccess) return e;
   const int per_sm = nst == kFxMaxSlots ? std::max(1, blocks(nw)) : 1;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(units, (int64_t)per_sm * num_sms()));
@@ -532,7 +532,7 @@ cudaError_t run_fx(const WorkItem* items, int n_items, int max_n, int S, const F
 }  // namespace
 
 bool fx_gemm_supported(int max_n) {
-  return max_n <= kFxMaxBlocks * kFxTile && FxSmem(max_n, 1).total(kFxFewWarps, 1) <= (size_t)kFxSmemCap;
+  return max_n <= kFxMaxBlocks * kFxTile && FxSmem(max_n, 1).total(kFxFewWarps, 1) <= kFxSmemCap;
 }
 
 cudaError_t launch_fx_quantize(const WorkItem* items, int n_items, const FxForm& A, int32_t* halves, cudaStream_t st) {
@@ -548,7 +548,7 @@ cudaError_t launch_fx_gemm(const WorkItem* items, int n_items, int max_n, double
   if (!fx_gemm_supported(max_n)) return cudaErrorInvalidValue;
   // columns per unit: the most that nrhs fills and shared memory holds
   int nc = nrhs > 4 ? 8 : nrhs > 2 ? 4 : nrhs;
-  while (nc > 1 && FxSmem(max_n, nc).total(kFxWarps, 1) > (size_t)kFxSmemCap) nc /= 2;
+  while (nc > 1 && FxSmem(max_n, nc).total(kFxWarps, 1) > kFxSmemCap) nc /= 2;
   // slices: so that the largest unit is at most an SM's share of the work, or
   // half of it at several columns, where the second reading of the tiles costs
   // nothing (216 operators of 343 rows on 152 SMs: 35 us with 1 slice and 43

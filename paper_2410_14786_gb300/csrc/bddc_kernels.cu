@@ -520,7 +520,7 @@ cudaError_t bgemv_t(const WorkItem* items, int n_items, int max_lda, const void*
   auto run = [&](auto kern, int nrb) -> cudaError_t {
     size_t sm = (size_t)max_lda * nrb * sizeof(Acc);
     if (sm > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      cudaError_t e = allow_smem(kern, sm);
       if (e != cudaSuccess) return e;
     }
     kern<<<n_items, kThreads, sm, st>>>(items, A, X, Y, yscatter, nrhs);
@@ -625,7 +625,7 @@ cudaError_t launch_phi_prolong(bddc_handle_s* h, const ApplyWork& W, int nrhs, c
   const dim3 grid(blocks, nrhs == 1 ? std::min(share, 2) : share, (nrhs + nb - 1) / nb);
   auto run = [&](auto kern, auto* pt) -> cudaError_t {
     if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      const cudaError_t e = allow_smem(kern, smem);
       if (e != cudaSuccess) return e;
     }
     kern<<<grid, kThreads, smem, st>>>(h->n_sub, nrhs, pt, h->d_pt_off, h->d_pt_ld, h->d_sub_goff, h->d_sub_coff,

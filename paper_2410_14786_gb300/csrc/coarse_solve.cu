@@ -1168,10 +1168,8 @@ cudaError_t build_sweeps(bddc_handle_s* h, const CoarseFactor& cf, SweepSet& S, 
       return e;
     const int smem = bl.max_front * (int)sizeof(double);
     if (smem > 48 * 1024) {
-      if ((e = cudaFuncSetAttribute(k_block_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-        return e;
-      if ((e = cudaFuncSetAttribute(k_block_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-        return e;
+      if ((e = allow_smem(k_block_fwd, smem)) != cudaSuccess) return e;
+      if ((e = allow_smem(k_block_bwd, smem)) != cudaSuccess) return e;
     }
   }
   if (!multi && !block) return cudaSuccess;

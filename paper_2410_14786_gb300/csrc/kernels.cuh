@@ -11,6 +11,17 @@
 
 namespace bddc {
 
+// Lets a kernel take `bytes` of dynamic shared memory. The limit that is set is
+// always the same (227 KB less some for the static arrays): it belongs to the
+// kernel, not to a launch, and one as small as this launch needs would refuse the
+// larger launch of another handle or thread.
+constexpr size_t kSmemMost = 225 * 1024;
+template <typename Kernel>
+inline cudaError_t allow_smem(Kernel kern, size_t bytes) {
+  if (bytes > kSmemMost) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost);
+}
+
 // z = M^-1 r for nrhs columns; all phases on `st`. prof_events, if not
 // null, holds 10 events recorded between the launches.
 // W: the work vectors to use (null: the handle's own).
