@@ -6,8 +6,8 @@
 // of GB300's float64 pipe, far below HBM. In fixed point a stored entry costs
 // 6 integer multiply-adds (3 for its row's and 3 for its column's product, 32
 // lanes per SM and clock), about half of the time its 8 bytes take from HBM, so
-// storing the triangle pays; at one column DRAM is 67 to 70 % busy and the integer
-// pipe 47 to 50 %, the rest the end of a unit, where every warp waits. From two columns
+// storing the triangle pays; at one column DRAM is 68 to 74 % busy and the integer
+// pipe 46 to 51 %, the rest the end of a unit, where every warp waits. From two columns
 // on the integer multiply-adds are the larger part (3 per full entry and column
 // against one float64 FMA at a sixteenth of their rate).
 //
