@@ -50,7 +50,7 @@ constexpr int kFxFewWarps = 8;
 constexpr int kFxTileBytes = kFxTileElems * 8;
 constexpr int kFxMaxSlots = 2;              // tiles in flight per warp
 constexpr size_t kFxSmemCap = kSmemMost;
-constexpr int kFxSmemSm = 228 * 1024;       // of an SM; 1 KB of it is taken by every block
+constexpr int kFxSmemSm = 228 * 1024;       // of an SM; every block takes 1 KB beside its own and the static arrays
 constexpr int kFarList = 256;
 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
@@ -504,7 +504,7 @@ cudaError_t run_fx(const WorkItem* items, int n_items, int max_n, int S, const F
   const FxUnits U{n_items, (nrhs + NC - 1) / NC, S};
   const int64_t units = (int64_t)n_items * U.ncb * S;
   auto fits = [&](int nw, int nst) { return L.total(nw, nst) <= kFxSmemCap; };
-  auto blocks = [&](int nw) { return std::min(kFxWarps / nw, (int)(kFxSmemSm / (L.total(nw, kFxMaxSlots) + 1024))); };
+  auto blocks = [&](int nw) { return std::min(kFxWarps / nw, (int)(kFxSmemSm / (L.total(nw, kFxMaxSlots) + 2048))); };
   // Warps of a block: as many as the largest operator has tiles, up to 12, in one
   // block per SM; narrower blocks, several to an SM, where there are more units than
   // SMs: the waits at a unit's end and its chain of loads then overlap with other
